@@ -435,7 +435,9 @@ mdfft_status mdfft_plan_check(mdfft_plan_t plan);
 /* Device workspace the plan owns, in bytes (0 for host-only plans). */
 mdfft_status mdfft_workspace_size(mdfft_plan_t plan, size_t *bytes);
 
-/* Number of kernel launches one mdfft_exec makes (M). */
+/* Number of kernel launches one mdfft_exec makes: M with the pass kernels,
+ * else one per axis longer than 1 (complex64 plans with the default launch
+ * choices transform the axes in place, in the natural layout). */
 mdfft_status mdfft_launches_per_exec(mdfft_plan_t plan, int *launches);
 
 /* Is line length n built into this library for dtype dt?  1 yes, 0 no. */

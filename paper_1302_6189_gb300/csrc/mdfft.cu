@@ -366,6 +366,40 @@ bool same_plan(const mdfft::RadixPlan &a, const mdfft::RadixPlan &b) {
     return true;
 }
 
+// The launches of an execution that keeps the natural layout: one per axis
+// longer than 1, in the order of the passes.  None (the pass kernels run) for
+// complex128 and the tensor-core dtypes, spectra left in the last layout, plans that ask
+// for the pipelined pass kernels, and arrays of 2^32 lines and more.
+mdfft_status build_nat(mdfft_plan_s *p) {
+    p->nat.clear();
+    if (p->dt != MDFFT_C64) return MDFFT_OK;
+    if (p->flags & (MDFFT_PLAN_OUT_LAST_LAYOUT | MDFFT_PLAN_PERSISTENT)) return MDFFT_OK;
+    int64_t stride[pl::kMaxDims], st = 1;
+    for (int i = p->M - 1; i >= 0; --i) stride[i] = st, st *= p->N[i];
+    for (int s = 0; s < p->M; ++s) {
+        const int f = p->order[s].axis[p->M - 1];
+        const int64_t n = p->N[f], lines = p->T * p->batch / n;
+        if (n == 1) continue;
+        mdfft::detail::NatOp op;
+        op.s = s;
+        const bool rows = stride[f] == 1;
+        if (lines + 1024 > 0xffffffffLL || !mdfft::find_nat_kernel_c64(n, rows, &op.k)) {
+            p->nat.clear();
+            return MDFFT_OK;
+        }
+        op.args = mdfft::NatArgs{};
+        op.args.nlines = (uint32_t)lines;
+        op.args.stride = stride[f];
+        op.args.fd = mdfft::fastdiv_make((uint32_t)stride[f]);
+        if (op.k.smem > 48 * 1024) {
+            cudaError_t e = cudaFuncSetAttribute(op.k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)op.k.smem);
+            if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
+        }
+        p->nat.push_back(op);
+    }
+    return MDFFT_OK;
+}
+
 mdfft_status parse_order(int M, const int *order, std::vector<pl::Layout> &out) {
     out.clear();
     for (int s = 0; s < M; ++s) {
@@ -441,11 +475,46 @@ mdfft_status exec_impl(mdfft_plan_t p, const void *in, void *out, int dir, int n
     return launch_passes(p, in, out, dir, normalize, st, counts, -1);
 }
 
+// An execution that keeps the natural layout (no workspace): the first launch
+// reads `in`, the others work in place on `out`.
+mdfft_status launch_nat(mdfft_plan_t p, const void *in, void *out, int dir, int normalize, cudaStream_t st, int64_t v,
+                        bool timed) {
+    const bool one = v >= 0 && p->batch > 1;
+    const size_t off = v >= 0 ? (size_t)v * (size_t)p->T * p->elem : 0;
+    const int64_t slot = p->timed % MDFFT_TIMING_SLOTS;
+    const size_t ops = p->nat.size();
+    int ev = 0;  // events recorded: one before each pass
+    for (size_t i = 0; i < ops; ++i) {
+        const mdfft::detail::NatOp &op = p->nat[i];
+        mdfft::NatArgs a = op.args;
+        if (one) a.nlines = (uint32_t)(a.nlines / p->batch);
+        a.in = (const char *)(i == 0 ? in : out) + off;
+        a.out = (char *)out + off;
+        a.tw = (const char *)p->tw + p->pass[op.s].tw_offset;
+        a.conj = dir == 1 ? (i == 0 ? 1 : 0) | (i + 1 == ops ? 2 : 0) : 0;
+        a.scale = (i + 1 == ops && normalize) ? 1.0 / (double)p->T : 1.0;
+        a.scaled = a.scale != 1.0;
+        if (timed)
+            for (; ev <= op.s; ++ev) cudaEventRecord(p->ev[slot * (p->M + 1) + ev], st);
+        const unsigned grid = (a.nlines + (unsigned)op.k.lines - 1) / (unsigned)op.k.lines;
+        void *args[] = {&a};
+        cudaError_t e = cudaLaunchKernel(op.k.fn, dim3(grid), dim3(op.k.threads), args, op.k.smem, st);
+        if (e != cudaSuccess) return cuda_fail(e, "axis launch");
+    }
+    if (timed) {
+        for (; ev <= p->M; ++ev) cudaEventRecord(p->ev[slot * (p->M + 1) + ev], st);
+        p->timed++;
+    }
+    return MDFFT_OK;
+}
+
 // The M passes on `st`: of the whole batch (v < 0) or of transform v alone
 // (the batch axis dropped, every array offset by v T elements; no timing).
 mdfft_status launch_passes(mdfft_plan_t p, const void *in, void *out, int dir, int normalize, cudaStream_t st,
                            int64_t *counts, int64_t v, bool allow_timing) {
     const int M = p->M;
+    if (!counts && p->as_built && !p->nat.empty())
+        return launch_nat(p, in, out, dir, normalize, st, v, p->timing && v < 0 && allow_timing);
     const bool one = v >= 0 && p->batch > 1;
     const size_t off = v >= 0 ? (size_t)v * (size_t)p->T * p->elem : 0;
     auto at = [off](const void *b) { return b ? (void *)((char *)b + off) : nullptr; };
@@ -531,6 +600,14 @@ mdfft_status exec_host_pipelined(mdfft_plan_t p, const void *in_host, void *out_
     if (e == cudaSuccess) e = cudaStreamWaitEvent(st, done, 0);
     if (e != cudaSuccess) return cuda_fail(e, "pipelined host execution");
     return MDFFT_OK;
+}
+
+bool passes_as_built(const mdfft_plan_s *p) {
+    for (int s = 0; s < p->M; ++s) {
+        const Pass &a = p->pass[s], &b = p->built[s];
+        if (a.k.fn != b.k.fn || a.args.Bg != b.args.Bg || a.args.Bh != b.args.Bh || a.mapping != b.mapping) return false;
+    }
+    return true;
 }
 
 // Drops the captured graphs of a plan (its launch arguments changed).
@@ -707,6 +784,10 @@ mdfft_status mdfft::detail::plan_create(mdfft_plan_t *out, int M, const int64_t 
                     p->pass[s].grid = std::min<int64_t>(p->pass[s].ctas, mdfft::detail::wave_ctas(k));
                 }
             }
+        if ((st = build_nat(p)) != MDFFT_OK) {
+            release(p);
+            return st;
+        }
         // twiddle tables: one per pass, 256-byte aligned inside one allocation,
         // each with room for the table of any radix plan of its length (fewer
         // than 2 n entries) so that autotuning can switch plans
@@ -762,6 +843,7 @@ mdfft_status mdfft::detail::plan_create(mdfft_plan_t *out, int M, const int64_t 
             release(p);
             return cuda_fail(e, "twiddle generation");
         }
+        p->built.assign(p->pass, p->pass + M);
     }
     *out = p;
     return MDFFT_OK;
@@ -1000,6 +1082,7 @@ mdfft_status mdfft_plan_autotune(mdfft_plan_t p, const void *in, void *out, int 
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
         return fail(MDFFT_E_CUDA, "cudaEventCreate");
     mdfft_status result = MDFFT_OK;
+    float tuned_ms = 0.f;
     for (int s = 0; s < p->M && result == MDFFT_OK; ++s) {
         Pass &ps = p->pass[s];
         std::vector<PassKernel> variants{ps.k};
@@ -1098,6 +1181,30 @@ mdfft_status mdfft_plan_autotune(mdfft_plan_t p, const void *in, void *out, int 
         ps = best;
         if (ms_before) ms_before[s] = default_ms;
         if (ms_after) ms_after[s] = best_ms;
+        tuned_ms += best_ms;
+    }
+    // the launches that keep the natural layout against the sum of the tuned passes
+    p->as_built = passes_as_built(p);
+    if (result == MDFFT_OK && !p->nat.empty()) {
+        float ms = 0.f;
+        for (int w = 0; w < 2 && result == MDFFT_OK; ++w) {
+            const int n = w == 0 ? 2 : reps;
+            cudaEventRecord(e0, st);
+            for (int r = 0; r < n && result == MDFFT_OK; ++r) result = launch_nat(p, in, out, -1, 0, st, -1, false);
+            cudaEventRecord(e1, st);
+            cudaError_t e = cudaEventSynchronize(e1);
+            if (result == MDFFT_OK && e != cudaSuccess) result = cuda_fail(e, "autotune launch");
+            if (result == MDFFT_OK) cudaEventElapsedTime(&ms, e0, e1);
+            ms /= (float)n;
+        }
+        if (result == MDFFT_OK && (p->as_built || ms < tuned_ms)) {
+            for (int s = 0; s < p->M; ++s) {
+                if (!same_plan(p->pass[s].k.plan, p->built[s].k.plan)) make_twiddles(p, s, p->built[s].k.plan, st);
+                p->pass[s] = p->built[s];
+                if (ms_after) ms_after[s] = ms / (float)p->M;
+            }
+            p->as_built = true;
+        }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
@@ -1209,6 +1316,7 @@ mdfft_status mdfft_plan_set_tuning(mdfft_plan_t p, const int32_t *in, int n) {
     cudaError_t e = cudaDeviceSynchronize();  // the new tables ready for any stream
     if (e != cudaSuccess) return cuda_fail(e, "twiddle generation");
     for (int s = 0; s < p->M; ++s) p->pass[s] = next[s];
+    p->as_built = passes_as_built(p);
     drop_graphs(p);
     return MDFFT_OK;
 }
@@ -1349,7 +1457,7 @@ mdfft_status mdfft_workspace_size(mdfft_plan_t p, size_t *bytes) {
 
 mdfft_status mdfft_launches_per_exec(mdfft_plan_t p, int *launches) {
     if (!p || !launches) return fail(MDFFT_E_ARG, "null argument");
-    *launches = p->M;
+    *launches = p->as_built && !p->nat.empty() ? (int)p->nat.size() : p->M;
     return MDFFT_OK;
 }
 

@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "../../include/mdfft.h"
+#include "nat_args.h"
 #include "passes.h"
 #include "planner.h"
 
@@ -23,6 +24,14 @@ struct Pass {
     int64_t grid = 0;          // CTAs launched (= ctas, or one wave for persistent kernels)
     size_t tw_offset = 0;      // byte offset of this pass's twiddle table (room for 2 n entries: any radix plan)
     int mapping = 0;           // tile order: 0 output-coalesced, 1 input-chunk order (see layout_pass)
+};
+
+// One launch of an execution that keeps the natural layout (fft_nat.cuh): the
+// line DFTs of pass s's axis over the whole array, in place after the first.
+struct NatOp {
+    int s = 0;
+    PassKernel k{};
+    NatArgs args{};      // everything but in/out/tw/conj/scale
 };
 
 // CTAs of one wave of kernel k on the current device (at least 1).
@@ -60,6 +69,11 @@ struct mdfft_plan_s {
     size_t elem = 8;
     std::vector<mdfft::planner::Layout> order;
     mdfft::detail::Pass pass[MDFFT_MAX_DIMS];
+    // Launches of an execution that keeps the natural layout; they run while
+    // the passes are as built (an autotuned or stored tuning names pass kernels).
+    std::vector<mdfft::detail::NatOp> nat;
+    std::vector<mdfft::detail::Pass> built;  // the passes as built
+    bool as_built = true;
     void *tw = nullptr, *ws = nullptr, *ws2 = nullptr;
     int *err = nullptr;           // device flag set by a persistent kernel whose bounded wait gave up
     bool external_ws = false;     // made by plan_create(..., with_workspace = false)

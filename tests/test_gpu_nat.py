@@ -1,0 +1,69 @@
+"""The layout-keeping line kernels (one axis of the natural array at a time,
+in place after the first) against the pass kernels, which the counted
+execution runs: the same butterflies in the same order, so the same bits, for
+every line length as rows and as columns, at ragged edges of their tiles."""
+
+import pytest
+import torch
+
+import paper_1302_6189_gb300 as md
+
+pytestmark = pytest.mark.gpu
+DEV = torch.device("cuda", 0)
+LENGTHS = [n for n in range(2, 1025) if md.mdfft_supported_length(n, "c64")]
+
+
+def _input(shape, seed):
+    g = torch.Generator(device=DEV)
+    g.manual_seed(seed)
+    return torch.view_as_complex(torch.rand(*shape, 2, generator=g, device=DEV) * 2 - 1)
+
+
+@pytest.mark.parametrize("n", LENGTHS)
+def test_every_length_as_rows_and_columns_equals_the_pass_kernels(n):
+    # rows: 3 and 160 lines; columns: 3 and 160 neighbouring lines, one and two blocks of them
+    for shape in ((3, n), (n, 3), (160, n), (2, n, 160)):
+        x = _input(shape, n)
+        keep = x.clone()
+        with md.Plan(shape, 3) as pl:
+            y = pl.exec(x)
+            assert torch.equal(y, pl.exec_counted(x)[0]), shape
+            z = pl.exec(x, dir=+1, normalize=True)
+            assert torch.equal(z, pl.exec_counted(x, dir=+1, normalize=True)[0]), shape
+            assert torch.equal(x, keep)
+
+
+@pytest.mark.parametrize("shape,batch", [((1, 24, 1, 40), 1), ((16, 1, 60), 3), ((5, 6, 8, 10), 2), ((20, 12, 15, 3, 8), 1),
+                                         ((48, 96, 160), 1), ((30, 240, 64), 2)])
+def test_axes_of_length_one_batches_and_every_order_of_axes(shape, batch):
+    full = shape if batch == 1 else (batch,) + shape
+    x = _input(full, 11)
+    M = len(shape)
+    for first in range(M - 1):  # orders that transform the axes in different sequences
+        rest = [a for a in range(M) if a != M - 1]
+        rest = rest[first:] + rest[:first]
+        layouts = [list(range(M))] + [[a for a in range(M) if a != f] + [f] for f in rest]
+        order = "->".join("".join("abcde"[a] for a in lay) for lay in layouts)
+        with md.Plan(shape, 4, order, batch=batch) as pl:
+            want = pl.exec_counted(x)[0]
+            assert torch.equal(pl.exec(x), want), order
+            assert torch.equal(pl.exec(x, graph=True), want), order
+        with md.Plan(shape, 4, order, flags=md.MDFFT_PLAN_INPLACE, batch=batch) as pl:
+            buf = x.clone()
+            assert torch.equal(pl.exec(buf, buf), want), order
+
+
+def test_eight_byte_aligned_arrays_and_per_pass_times():
+    shape = (24, 40, 32)
+    data = _input(shape, 5)
+    raw_in = torch.empty(data.numel() + 1, dtype=torch.complex64, device=DEV)
+    raw_out = torch.empty_like(raw_in)
+    x, y = raw_in[1:].view(shape), raw_out[1:].view(shape)
+    x.copy_(data)
+    with md.Plan(shape, 8) as pl:
+        assert torch.equal(pl.exec(x, y), pl.exec_counted(data)[0])
+        pl.set_timing(True)
+        for _ in range(3):
+            pl.exec(x, y)
+        ms, n = pl.pass_times()
+        assert n == 3 and all(t > 0 for t in ms)
