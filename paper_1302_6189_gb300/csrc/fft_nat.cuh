@@ -191,6 +191,15 @@ __device__ __forceinline__ double2 ld_cached(const double2 *p) {
     return v;
 }
 
+// The launches of an execution follow each other by programmatic dependence:
+// the next one may be set up while this one runs, and waits here until this
+// one is complete and its stores are visible.  (60 x 240 x 160: 28.7 -> 22.8 us
+// for three launches, 24^5 87.1 -> 77.9 us for five, 256^3 130 -> 122.6 us.)
+__device__ __forceinline__ void follow_previous_launch() {
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
 template <typename C, int SIZE> __device__ __forceinline__ void conj_all(C (&v)[SIZE]) {
 #pragma unroll
     for (int r = 0; r < SIZE; ++r) v[r].y = -v[r].y;
@@ -293,6 +302,7 @@ __global__ void __launch_bounds__(ColCfg<Real, N>::THREADS) fft_nat_col_kernel(c
     const uint32_t o = fastdiv(l, a.fd);
     const int64_t base = (int64_t)o * N * a.stride + (l - o * a.fd.d);
     const C *tw = reinterpret_cast<const C *>(a.tw);
+    follow_previous_launch();
     if constexpr (Cfg::parts.n > 1) {  // twiddles to shared memory; the barrier after the first part covers them
         C *stw = buf + N * CC::COLS;
         for (int q = tid; q < tw_entries(Cfg::plan); q += CC::THREADS) stw[q] = __ldg(tw + q);
@@ -428,6 +438,7 @@ __global__ void __launch_bounds__(RowCfg<Real, N>::THREADS, RowCfg<Real, N>::MIN
     const C *in = reinterpret_cast<const C *>(a.in), *tw = reinterpret_cast<const C *>(a.tw);
     C *out = reinterpret_cast<C *>(a.out);
     const int tid = threadIdx.x;
+    follow_previous_launch();
     if constexpr (Cfg::parts.n == 1) {
         // one thread per line: a warp copies its 32 lines (contiguous in
         // memory) through its own rows of shared memory, in and out
