@@ -454,21 +454,18 @@ mdfft_status mdfft_destroy(mdfft_plan_t plan);
  * in flight, and a CUDA graph per table slot.  mdfft_server_step() admits
  * queued requests first come first served while the HBM budget (each request
  * is charged input + output + workspace = 3 T 8 bytes) and the slot count
- * allow, then launches -- as one graph launch of one persistent kernel -- the
- * next pass of every request in flight, whatever its shape.  A request that
- * arrives while others are on the GPU joins at the next step; it leaves after
- * its last pass.  Requests advance one pass per step, so a step has no
- * dependencies inside it and nothing waits on the device.  At low load --
- * no request queued and at most `direct` requests with passes left
+ * allow, then launches -- as one graph launch -- the next axis of every
+ * request in flight, whatever its shape, in the order of the plan's passes.  A
+ * request that arrives while others are on the GPU joins at the next step; it
+ * leaves after its last axis.  Requests advance one axis per step, so a step
+ * has no dependencies inside it and nothing waits on the device.  At low load --
+ * no request queued and at most `direct` requests with axes left
  * (mdfft_server_set_direct, default 4) -- a step instead launches every
- * remaining pass of those requests, oldest first, as plain pass launches
- * (those of mdfft_exec): a lone request then runs its passes back to back
- * instead of one per step.  Line lengths
- * 16, 24, 32, 48, 64, 96, 128, 160, 192, 256 run inside the persistent
- * kernel; passes of 16 to 64 points whose arrays are 16-byte aligned go
- * instead to a second persistent kernel of the same graph, launched after
- * it, that runs one thread per line with every radix stage in registers
- * (mdfft_server_set_line_kernel); other supported lengths run as separate
+ * remaining axis of those requests, oldest first, as plain launches (those of
+ * mdfft_exec): a lone request then runs its axes back to back instead of one
+ * per step.  Line lengths 16, 24, 32, 48, 64, 96, 128, 160, 192, 256 have
+ * a kernel each for rows and for columns in the step's graph; a step runs the
+ * ones it has work for as parallel branches.  Other supported lengths run as separate
  * launches in the same step.  Results are the same as mdfft_exec's for the
  * same shape (the same radix plans and butterflies in the same order).  All work goes to `stream`; the caller's buffers must stay valid
  * until the request is done.  Errors: E_ARG, E_RANGE (request above the
@@ -481,7 +478,7 @@ typedef struct {
     int64_t steps, graph_launches, kernel_launches;
     int64_t inflight, queued;
     size_t bytes_in_use, budget_bytes;
-    int grid_ctas; /* CTAs of the persistent kernel */
+    int grid_ctas; /* CTAs of a step's kernel at most: the widest one's resident wave, or what set_grid gave */
     int64_t cancelled;
     int64_t direct_requests; /* requests whose remaining passes ran as plain launches (low load) */
 } mdfft_server_stats;
@@ -517,7 +514,8 @@ mdfft_status mdfft_server_cancel(mdfft_server_t s, int64_t request_id);
 mdfft_status mdfft_server_drain(mdfft_server_t s);
 /* Sets the server clock's zero to now (records an event on the stream and waits for it). */
 mdfft_status mdfft_server_reset_clock(mdfft_server_t s);
-/* Re-captures the graphs with a persistent grid of `ctas` CTAs (autotuning). */
+/* At most `ctas` CTAs for each kernel of a step (default: one resident wave of
+ * each); a kernel's CTAs walk its tiles.  Waits for the steps in flight. */
 mdfft_status mdfft_server_set_grid(mdfft_server_t s, int ctas);
 /* Steps in flight on the GPU at most (1..8, default 2): a batched step is
  * launched only while fewer are outstanding, so requests arriving meanwhile
@@ -525,7 +523,7 @@ mdfft_status mdfft_server_set_grid(mdfft_server_t s, int ctas);
  * direct steps are held back only while batched steps are in flight). */
 mdfft_status mdfft_server_set_depth(mdfft_server_t s, int depth);
 /* At most this many consecutive tiles (1..64, default 4) are dealt to a CTA
- * of the persistent kernel at a time; each step deals chunks of its tile
+ * of a step's kernel at a time; each kernel deals chunks of its tile
  * count / grid, between 1 and this maximum, so that small steps still use
  * every CTA.  Larger chunks mean fewer item lookups, smaller ones evener
  * load.  Results do not depend on it. */
@@ -535,10 +533,8 @@ mdfft_status mdfft_server_set_chunk(mdfft_server_t s, int chunk);
  * remaining passes directly, oldest request first.  Results do not depend on
  * it. */
 mdfft_status mdfft_server_set_direct(mdfft_server_t s, int max_requests);
-/* 1 (default): passes of 16 to 64 points with 16-byte aligned arrays run in
- * the line kernel of the step; 0: in the grouped persistent kernel like the
- * other lengths.  Takes effect at the next step; results do not depend on
- * it.  E_ARG unless enable is 0 or 1. */
+/* Kept for programs that call it: every length has a kernel of its own in the
+ * step, so 0 and 1 run the same.  E_ARG unless enable is 0 or 1. */
 mdfft_status mdfft_server_set_line_kernel(mdfft_server_t s, int enable);
 mdfft_status mdfft_server_get_stats(mdfft_server_t s, mdfft_server_stats *out);
 mdfft_status mdfft_server_destroy(mdfft_server_t s);

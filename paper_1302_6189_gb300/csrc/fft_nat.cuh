@@ -204,6 +204,10 @@ template <typename C, int SIZE> __device__ __forceinline__ void conj_all(C (&v)[
 #pragma unroll
     for (int r = 0; r < SIZE; ++r) v[r].y = -v[r].y;
 }
+template <typename C, int SIZE> __device__ __forceinline__ void zero_all(C (&v)[SIZE]) {
+#pragma unroll
+    for (int r = 0; r < SIZE; ++r) v[r] = C{0, 0};
+}
 // conjugation and scale of the last pass, as store_tile applies them
 template <typename C, int SIZE> __device__ __forceinline__ void finish_all(C (&v)[SIZE], const NatArgs &a) {
     using Real = decltype(v[0].x);
@@ -261,10 +265,14 @@ template <typename Real, int N, int PI> struct ColParts {
 #pragma unroll
                     for (int r = 0; r < SIZE; ++r) v[i][r] = ld_stream(p + (int64_t)(r * D) * a.stride);
                     if (a.conj & 1) conj_all(v[i]);
+                } else {  // (defined values: left alone, they would stay live around a loop over tiles)
+                    zero_all(v[i]);
                 }
             } else if (live) {
 #pragma unroll
                 for (int r = 0; r < SIZE; ++r) v[i][r] = buf[(at[i] + r * D) * COLS + col];
+            } else {
+                zero_all(v[i]);
             }
         }
 #pragma unroll
@@ -289,6 +297,16 @@ template <typename Real, int N, int PI> struct ColParts {
     }
 };
 
+// Lines l0 .. l0 + COLS - 1 by the whole CTA (tw: the twiddles, staged when the length has an exchange).
+template <typename Real, int N, typename C = typename Cx<Real>::T>
+__device__ __forceinline__ void nat_col_tile(const C *in, C *out, C *buf, const C *tw, int tid, uint32_t l0, const NatArgs &a) {
+    using CC = ColCfg<Real, N>;
+    const int col = tid % CC::COLS, t = tid / CC::COLS;
+    const uint32_t l = l0 + col, o = fastdiv(l, a.fd);
+    const int64_t base = (int64_t)o * N * a.stride + (l - o * a.fd.d);
+    ColParts<Real, N, 0>::run(in + base, out + base, buf, tw, col, t, l < a.nlines, a);
+}
+
 template <typename Real, int N>
 __global__ void __launch_bounds__(ColCfg<Real, N>::THREADS) fft_nat_col_kernel(const NatArgs a) {
     using CC = ColCfg<Real, N>;
@@ -296,11 +314,7 @@ __global__ void __launch_bounds__(ColCfg<Real, N>::THREADS) fft_nat_col_kernel(c
     using C = typename Cfg::C;
     extern __shared__ __align__(16) unsigned char nat_smem[];
     C *buf = reinterpret_cast<C *>(nat_smem);
-    const int tid = threadIdx.x, col = tid % CC::COLS, t = tid / CC::COLS;
-    const uint32_t l = blockIdx.x * CC::COLS + col;
-    const bool ok = l < a.nlines;
-    const uint32_t o = fastdiv(l, a.fd);
-    const int64_t base = (int64_t)o * N * a.stride + (l - o * a.fd.d);
+    const int tid = threadIdx.x;
     const C *tw = reinterpret_cast<const C *>(a.tw);
     follow_previous_launch();
     if constexpr (Cfg::parts.n > 1) {  // twiddles to shared memory; the barrier after the first part covers them
@@ -309,8 +323,7 @@ __global__ void __launch_bounds__(ColCfg<Real, N>::THREADS) fft_nat_col_kernel(c
         tw = stw;
         if constexpr (Cfg::parts.count[0] > 1) __syncthreads();
     }
-    ColParts<Real, N, 0>::run(reinterpret_cast<const C *>(a.in) + base, reinterpret_cast<C *>(a.out) + base, buf, tw,
-                              col, t, ok, a);
+    nat_col_tile<Real, N>(reinterpret_cast<const C *>(a.in), reinterpret_cast<C *>(a.out), buf, tw, tid, blockIdx.x * CC::COLS, a);
 }
 
 // ------------------------------------------------------------------ rows
@@ -395,7 +408,10 @@ template <typename Real, int N, int PI> struct RowParts {
             live[i] = line[i] < have;
             k[i] = (int)((unsigned)b % (unsigned)B);
             at[i] = digits_place<N, STAGES>(k[i]) * (N / B) + (int)((unsigned)b / (unsigned)B);
-            if (!live[i]) continue;
+            if (!live[i]) {
+                zero_all(v[i]);
+                continue;
+            }
             if constexpr (FIRST) {
                 const C *src = in + line[i] * N + at[i];
 #pragma unroll
@@ -428,22 +444,16 @@ template <typename Real, int N, int PI> struct RowParts {
     }
 };
 
-template <typename Real, int N>
-__global__ void __launch_bounds__(RowCfg<Real, N>::THREADS, RowCfg<Real, N>::MINB) fft_nat_row_kernel(const NatArgs a) {
+// Lines l0 .. l0 + LINES - 1 by the whole CTA.
+template <typename Real, int N, typename C = typename Cx<Real>::T>
+__device__ __forceinline__ void nat_row_tile(const C *in, C *out, C *buf, const C *tw, int tid, uint32_t l0, const NatArgs &a) {
     using RC = RowCfg<Real, N>;
     using Cfg = NatCfg<Real, N, true>;
-    using C = typename Cfg::C;
-    extern __shared__ __align__(16) unsigned char nat_smem[];
-    C *buf = reinterpret_cast<C *>(nat_smem);
-    const C *in = reinterpret_cast<const C *>(a.in), *tw = reinterpret_cast<const C *>(a.tw);
-    C *out = reinterpret_cast<C *>(a.out);
-    const int tid = threadIdx.x;
-    follow_previous_launch();
     if constexpr (Cfg::parts.n == 1) {
         // one thread per line: a warp copies its 32 lines (contiguous in
         // memory) through its own rows of shared memory, in and out
         const int lane = tid & 31;
-        const uint32_t l0 = blockIdx.x * RC::LINES + (tid - lane);
+        l0 += tid - lane;
         if (l0 >= a.nlines) return;  // (whole warps; no CTA barrier below)
         const int have = (int)(a.nlines - l0 < 32 ? a.nlines - l0 : 32) * N;
         C *rows = buf + (tid - lane) * RC::RS, *row = rows + lane * RC::RS;
@@ -469,11 +479,19 @@ __global__ void __launch_bounds__(RowCfg<Real, N>::THREADS, RowCfg<Real, N>::MIN
             if (e < have) out[base + e] = rows[e / N * RC::RS + e % N];
         }
     } else {
-        const uint32_t l0 = blockIdx.x * RC::LINES;
         const int64_t base = (int64_t)l0 * N;
         const uint32_t left = a.nlines - l0;
         RowParts<Real, N, 0>::run(in + base, out + base, buf, tw, tid, left < RC::LINES ? (int)left : RC::LINES, a);
     }
+}
+
+template <typename Real, int N>
+__global__ void __launch_bounds__(RowCfg<Real, N>::THREADS, RowCfg<Real, N>::MINB) fft_nat_row_kernel(const NatArgs a) {
+    using C = typename Cx<Real>::T;
+    extern __shared__ __align__(16) unsigned char nat_smem[];
+    follow_previous_launch();
+    nat_row_tile<Real, N>(reinterpret_cast<const C *>(a.in), reinterpret_cast<C *>(a.out), reinterpret_cast<C *>(nat_smem),
+                          reinterpret_cast<const C *>(a.tw), threadIdx.x, blockIdx.x * RowCfg<Real, N>::LINES, a);
 }
 
 }  // namespace mdfft

@@ -314,6 +314,20 @@ int64_t mdfft::detail::wave_ctas(const PassKernel &k) {
     return (int64_t)sms * std::max(per, 1);
 }
 
+cudaError_t mdfft::detail::launch_following(const PassKernel &k, unsigned grid, void **args, cudaStream_t st) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3((unsigned)k.threads);
+    cfg.dynamicSmemBytes = k.smem;
+    cfg.stream = st;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelExC(&cfg, k.fn, args);
+}
+
 void mdfft::detail::retile_pass(const mdfft_plan_s *p, int s, int lines, PassArgs *out, int64_t *ctas) {
     const Pass &ps = p->pass[s];
     PassArgs a = ps.args;
@@ -475,22 +489,6 @@ mdfft_status exec_impl(mdfft_plan_t p, const void *in, void *out, int dir, int n
     return launch_passes(p, in, out, dir, normalize, st, counts, -1);
 }
 
-// Launches a kernel that may be set up while the launch before it on the
-// stream still runs (the kernel itself waits for that one's completion).
-cudaError_t launch_following(const PassKernel &k, unsigned grid, void **args, cudaStream_t st) {
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr.val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3((unsigned)k.threads);
-    cfg.dynamicSmemBytes = k.smem;
-    cfg.stream = st;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelExC(&cfg, k.fn, args);
-}
-
 // An execution that keeps the natural layout (no workspace): the first launch
 // reads `in`, the others work in place on `out`.
 mdfft_status launch_nat(mdfft_plan_t p, const void *in, void *out, int dir, int normalize, cudaStream_t st, int64_t v,
@@ -514,7 +512,7 @@ mdfft_status launch_nat(mdfft_plan_t p, const void *in, void *out, int dir, int 
             for (; ev <= op.s; ++ev) cudaEventRecord(p->ev[slot * (p->M + 1) + ev], st);
         const unsigned grid = (a.nlines + (unsigned)op.k.lines - 1) / (unsigned)op.k.lines;
         void *args[] = {&a};
-        cudaError_t e = launch_following(op.k, grid, args, st);
+        cudaError_t e = mdfft::detail::launch_following(op.k, grid, args, st);
         if (e != cudaSuccess) return cuda_fail(e, "axis launch");
     }
     if (timed) {

@@ -37,6 +37,10 @@ struct NatOp {
 // CTAs of one wave of kernel k on the current device (at least 1).
 int64_t wave_ctas(const PassKernel &k);
 
+// Launches a kernel that may be set up while the launch before it on the
+// stream still runs (the kernel itself waits for that one's completion).
+cudaError_t launch_following(const PassKernel &k, unsigned grid, void **args, cudaStream_t st);
+
 // Records the message for mdfft_last_error() on this thread; returns st.
 mdfft_status fail(mdfft_status st, const std::string &msg);
 mdfft_status cuda_fail(cudaError_t e, const char *what);

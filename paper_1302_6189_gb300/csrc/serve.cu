@@ -1,20 +1,21 @@
 // serve.cu -- batched serving of M-D FFT requests of different shapes.
 //
-// Continuous batching at pass granularity.  Every step launches, in one
-// persistent kernel, the next pass (Fig. 4 step + transpose, as in
-// mdfft_exec) of every request in flight, whatever its shape; a request that
-// arrives while others are on the GPU joins at the next step, as soon as the
-// HBM budget and a slot allow, and leaves after its last pass.  One step is
-// one launch of a CUDA graph (copy of the step's work table from pinned host
-// memory, then the persistent kernel), captured once per table slot.  The
-// persistent kernel walks the tiles of all items with a grid stride; a CTA
-// finds the item of a tile by binary search over the items' first tiles and
-// runs the tile code of that item's line length.  Passes of lines of 16 to
-// 64 points (16-byte aligned arrays) go instead to a second persistent
-// kernel of the same graph, launched after the first, whose warps each take
-// whole 32-line tiles and run the one-thread-per-line code of fft_line.cuh.
-// There is no device-side waiting: passes of one request are in consecutive
-// steps, ordered by the stream.
+// Continuous batching at pass granularity.  Every step launches the next axis
+// (in the order of the plan's passes) of every request in flight, whatever its
+// shape; a request that arrives while others are on the GPU joins at the next
+// step, as soon as the HBM budget and a slot allow, and leaves after its last
+// axis.  One step is one launch of a CUDA graph: the copy of the step's work
+// table from pinned host memory, then one kernel per line length and kind
+// (rows or columns, fft_nat.cuh) that has work, as parallel branches, so that
+// the tail of one overlaps the others.  The graph of a table slot is made
+// once; a step enables the kernels it needs and sets their grids.
+//
+// A kernel per length, and not one persistent kernel with all lengths in a
+// switch: that one ran every length at the registers and the shared memory of
+// the longest (64 registers, 4 CTAs per SM), staged the twiddles per tile and
+// closed every tile with four CTA barriers; the 100-request mix moved its data
+// at half the copy rate.  There is no device-side waiting: the axes of one
+// request are in consecutive steps, ordered by the stream.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -26,9 +27,10 @@
 #include <unordered_map>
 #include <vector>
 
-#include "fft_line.cuh"
+#include "fft_nat.cuh"
 #include "plan_internal.h"
 
+using mdfft::NatArgs;
 using mdfft::PassArgs;
 using mdfft::detail::cuda_fail;
 using mdfft::detail::fail;
@@ -36,92 +38,33 @@ using mdfft::detail::fail;
 namespace mdfft {
 namespace serve {
 
-constexpr int kMaxItems = 512;  // passes per step
+constexpr int kMaxItems = 512;  // axes per step (one per request)
 constexpr int kSlots = 8;       // tables (and graphs) in flight
-constexpr int kThreads = 256;   // CTA size of the persistent kernel (every length uses all of it)
 
-// line lengths the persistent kernel carries (complex64); other lengths run
-// as separate launches of their own pass kernel within the same step
+// line lengths with a kernel in the step's graph (complex64); other lengths
+// run as launches of their own within the same step
 #define MDFFT_SERVE_LENGTHS(X) X(0, 16) X(1, 24) X(2, 32) X(3, 48) X(4, 64) X(5, 96) X(6, 128) X(7, 160) X(8, 192) X(9, 256)
 #define MDFFT_COUNT_KIND(i, N) +1
 constexpr int kKinds = 0 MDFFT_SERVE_LENGTHS(MDFFT_COUNT_KIND);
 #undef MDFFT_COUNT_KIND
 static_assert(kKinds == 10, "serving kinds are numbered 0 .. kKinds - 1 in MDFFT_SERVE_LENGTHS");
+constexpr int kGroups = 2 * kKinds;  // group 2 kind: columns, 2 kind + 1: rows
 
 struct Item {
-    PassArgs args;
-    int64_t start;  // first tile of this item in the step's tile numbering
-    int kind;       // index into MDFFT_SERVE_LENGTHS
-    int pad;
+    NatArgs args;
+    int64_t start;  // first tile of this item in its group's numbering
+};
+
+struct Group {
+    int first, n;   // items[first, first + n)
+    int chunk;      // consecutive tiles dealt to a CTA at a time
+    int64_t total;  // tiles
 };
 
 struct Table {
-    int n;          // items of the grouped kernel: items[0, n)
-    int chunk;      // consecutive tiles dealt to a CTA at a time
-    int64_t total;  // tiles in the step
-    // items of the line kernels, group g after those of the groups before:
-    // items[n + n_line[0] + .. + n_line[g-1], + n_line[g]), tiles numbered from 0 in each group
-    int n_line[2];
-    int chunk_line[2];  // consecutive 32-line tiles dealt to a warp at a time
-    int64_t total_line[2];
+    Group group[kGroups];
     Item items[kMaxItems];
 };
-
-// line lengths of the one-thread-per-line serving kernels: kind kLineKind + i;
-// group 0 (16, 24, 32: up to 90 registers a thread in the standalone
-// kernel) and group 1 (48, 64: up to 190) are separate kernels, so that the
-// short lengths keep more warps per SM
-#define MDFFT_SERVE_LINE_LENGTHS(X) X(0, 16) X(1, 24) X(2, 32) X(3, 48) X(4, 64)
-#define MDFFT_SERVE_LINE_GROUP0(X) X(0, 16) X(1, 24) X(2, 32)
-#define MDFFT_SERVE_LINE_GROUP1(X) X(3, 48) X(4, 64)
-constexpr int kLineKind = 100;
-constexpr int kLineThreads = 128, kLineWarps = kLineThreads / 32;
-constexpr int line_group(int kind) { return kind - kLineKind >= 3 ? 1 : 0; }
-constexpr size_t kArgsBytes = (sizeof(PassArgs) + 15) / 16 * 16;
-constexpr size_t cmax2(size_t a, size_t b) { return a > b ? a : b; }
-#define MDFFT_LINE_RS_MAX(i, N) cmax2((size_t)LineCfg<N>::RS,
-#define MDFFT_LINE_CLOSE(i, N) )
-// staging row stride of each group: its longest line's
-constexpr size_t kLineRs[2] = {MDFFT_SERVE_LINE_GROUP0(MDFFT_LINE_RS_MAX) 0 MDFFT_SERVE_LINE_GROUP0(MDFFT_LINE_CLOSE),
-                               MDFFT_SERVE_LINE_GROUP1(MDFFT_LINE_RS_MAX) 0 MDFFT_SERVE_LINE_GROUP1(MDFFT_LINE_CLOSE)};
-// per warp: the item's arguments, 32 staging rows, 32 line offsets
-constexpr size_t line_warp_smem(int g) { return kArgsBytes + 32 * kLineRs[g] * sizeof(float2) + 32 * sizeof(int64_t); }
-constexpr size_t kLineSmem[2] = {kLineWarps * line_warp_smem(0), kLineWarps * line_warp_smem(1)};
-
-int line_kind_of(int64_t n) {
-    switch (n) {
-#define MDFFT_KIND(i, N) \
-    case N:              \
-        return kLineKind + i;
-        MDFFT_SERVE_LINE_LENGTHS(MDFFT_KIND)
-#undef MDFFT_KIND
-        default:
-            return -1;
-    }
-}
-
-template <int N> using ServeCfg = PassCfg<float, N, 0, kThreads>;
-template <int N> constexpr size_t smem_of() { return ServeCfg<N>::SMEM; }
-template <int N> constexpr int threads_of() { return ServeCfg<N>::THREADS; }
-constexpr size_t cmax(size_t a, size_t b) { return a > b ? a : b; }
-#define MDFFT_SMEM_MAX(i, N) cmax(smem_of<N>(),
-#define MDFFT_CLOSE(i, N) )
-constexpr size_t kSmem = MDFFT_SERVE_LENGTHS(MDFFT_SMEM_MAX) 0 MDFFT_SERVE_LENGTHS(MDFFT_CLOSE);
-#define MDFFT_THR_OK(i, N) static_assert(threads_of<N>() <= kThreads, "serve CTA too small");
-MDFFT_SERVE_LENGTHS(MDFFT_THR_OK)
-
-// tile lines of the serving configuration of each kind
-int lines_of_kind(int kind) {
-    switch (kind) {
-#define MDFFT_LINES(i, N) \
-    case i:               \
-        return ServeCfg<N>::LINES;
-        MDFFT_SERVE_LENGTHS(MDFFT_LINES)
-#undef MDFFT_LINES
-        default:
-            return 0;
-    }
-}
 
 int kind_of(int64_t n) {
     switch (n) {
@@ -135,79 +78,52 @@ int kind_of(int64_t n) {
     }
 }
 
-__global__ void __launch_bounds__(kThreads, 4) serve_kernel(const Table *tab) {
-    extern __shared__ __align__(16) unsigned char smem[];
-    __shared__ PassArgs args;
-    const int n = tab->n;
-    const int64_t total = tab->total;
-    // chunks of kChunk consecutive tiles, dealt to the CTAs in turn: tiles of
-    // different line lengths even out across CTAs, and consecutive tiles of
-    // a chunk mostly belong to one item, so item lookups and argument copies
-    // are rare (items are in increasing tile order, so lookups only advance)
-    const int kChunk = tab->chunk;
-    int cur = 0;
-    int64_t cur_start = 0, cur_end = n > 1 ? tab->items[1].start : total;  // item 0 starts at tile 0
-    int kind = -1;
-    for (int64_t c0 = (int64_t)blockIdx.x * kChunk; c0 < total; c0 += (int64_t)gridDim.x * kChunk)
-        for (int64_t t = c0; t < c0 + kChunk && t < total; ++t) {
-        if (t >= cur_end || kind < 0) {
-            if (t >= cur_end) {  // binary search over the items after cur: last one starting <= t
-                int lo = cur + 1, hi = n - 1;
-                while (lo < hi) {
-                    const int mid = (lo + hi + 1) >> 1;
-                    if (tab->items[mid].start <= t) lo = mid;
-                    else hi = mid - 1;
-                }
-                cur = lo;
-                cur_start = tab->items[cur].start;
-                cur_end = cur + 1 < n ? tab->items[cur + 1].start : total;
-            }
-            __syncthreads();  // every thread is done with the previous arguments
-            const int *src = reinterpret_cast<const int *>(&tab->items[cur].args);
-            int *dst = reinterpret_cast<int *>(&args);
-            for (int w = threadIdx.x; w < (int)(sizeof(PassArgs) / sizeof(int)); w += blockDim.x) dst[w] = src[w];
-            kind = tab->items[cur].kind;
-            __syncthreads();
-        }
-        const int64_t local = t - cur_start;
-        switch (kind) {
-#define MDFFT_RUN(i, N)                                                  \
-    case i:                                                              \
-        pass_tile<float, N, 0, kThreads>(args, local, smem, threadIdx.x); \
-        break;
-            MDFFT_SERVE_LENGTHS(MDFFT_RUN)
-#undef MDFFT_RUN
-            default:
-                break;
-        }
-        __syncthreads();  // shared memory is reused by the next tile
-    }
+// index of a length in MDFFT_SERVE_LENGTHS
+template <int N> constexpr int kKindOf = [] {
+    int k = -1;
+#define MDFFT_KIND(i, n) k = N == n ? i : k;
+    MDFFT_SERVE_LENGTHS(MDFFT_KIND)
+#undef MDFFT_KIND
+    return k;
+}();
+
+template <int N, bool ROWS> constexpr int axis_threads() { return ROWS ? RowCfg<float, N>::THREADS : ColCfg<float, N>::THREADS; }
+// 40 warps per SM (48 registers; 72 with a whole line in registers)
+template <int N, bool ROWS> constexpr int axis_min_ctas() {
+    return (NatCfg<float, N, ROWS>::parts.n == 1 ? 896 : 1280) / axis_threads<N, ROWS>();
 }
 
-// A line kernel (group G): warp w of the grid takes chunks of
-// chunk_line[G] consecutive 32-line tiles of the group's items in turn; it
-// copies an item's arguments to its own shared memory when it reaches the
-// item's tiles (items are in increasing tile order, so lookups only
-// advance).  No CTA barrier.  Registers: group 0 fits 4 CTAs per SM, group 1 2.
-template <int G>
-__global__ void __launch_bounds__(kLineThreads, G == 0 ? 4 : 2) serve_line_kernel(const Table *tab) {
-    extern __shared__ __align__(16) unsigned char line_smem[];
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    unsigned char *wsm = line_smem + warp * line_warp_smem(G);
-    PassArgs &args = *reinterpret_cast<PassArgs *>(wsm);
-    float2 *stage = reinterpret_cast<float2 *>(wsm + kArgsBytes);
-    int64_t *lbase = reinterpret_cast<int64_t *>(stage + 32 * kLineRs[G]);
-    const Item *items = tab->items + tab->n + (G == 1 ? tab->n_line[0] : 0);
-    const int n = tab->n_line[G];
-    const int64_t total = tab->total_line[G];
-    const int64_t chunk = tab->chunk_line[G];
-    const int64_t gw = (int64_t)blockIdx.x * kLineWarps + warp, nw = (int64_t)gridDim.x * kLineWarps;
-    int cur = -1, kind = -1;
+// A group's tiles: chunks of consecutive tiles dealt to the CTAs in turn.
+// Consecutive tiles mostly belong to one item, so item lookups and argument
+// copies are rare (items are in increasing tile order: lookups only advance).
+// The twiddles of a length are the same in every plan: columns stage them once
+// per CTA.
+template <int N, bool ROWS>
+__global__ void __launch_bounds__(axis_threads<N, ROWS>(), axis_min_ctas<N, ROWS>()) serve_axis_kernel(const Table *tab) {
+    using CC = ColCfg<float, N>;
+    using RC = RowCfg<float, N>;
+    using Cfg = NatCfg<float, N, ROWS>;
+    constexpr int LINES = ROWS ? RC::LINES : CC::COLS, THREADS = ROWS ? RC::THREADS : CC::THREADS;
+    extern __shared__ __align__(16) unsigned char serve_smem[];
+    __shared__ NatArgs a;
+    float2 *buf = reinterpret_cast<float2 *>(serve_smem);
+    const Group &g = tab->group[2 * kKindOf<N> + (ROWS ? 1 : 0)];
+    const Item *items = tab->items + g.first;
+    const int n = g.n, chunk = g.chunk, tid = threadIdx.x;
+    const int64_t total = g.total;
+    const float2 *tw = reinterpret_cast<const float2 *>(items[0].args.tw);
+    if constexpr (!ROWS && Cfg::parts.n > 1) {
+        float2 *stw = buf + N * CC::COLS;
+        for (int q = tid; q < tw_entries(Cfg::plan); q += THREADS) stw[q] = __ldg(tw + q);
+        tw = stw;
+    }
+    int cur = -1;
     int64_t cur_start = 0, cur_end = 0;
-    for (int64_t c0 = gw * chunk; c0 < total; c0 += nw * chunk)
+    for (int64_t c0 = (int64_t)blockIdx.x * chunk; c0 < total; c0 += (int64_t)gridDim.x * chunk)
         for (int64_t t = c0; t < c0 + chunk && t < total; ++t) {
-            if (t >= cur_end) {  // the last item after cur starting at or before t
-                int lo = cur + 1, hi = n - 1;
+            __syncthreads();  // shared memory of the previous tile is free
+            if (t >= cur_end) {
+                int lo = cur + 1, hi = n - 1;  // the last item after cur starting at or before t
                 while (lo < hi) {
                     const int mid = (lo + hi + 1) >> 1;
                     if (items[mid].start <= t) lo = mid;
@@ -216,33 +132,46 @@ __global__ void __launch_bounds__(kLineThreads, G == 0 ? 4 : 2) serve_line_kerne
                 cur = lo;
                 cur_start = items[cur].start;
                 cur_end = cur + 1 < n ? items[cur + 1].start : total;
-                __syncwarp();  // every lane is done with the previous arguments
                 const int *src = reinterpret_cast<const int *>(&items[cur].args);
-                int *dst = reinterpret_cast<int *>(&args);
-                for (int w = lane; w < (int)(sizeof(PassArgs) / sizeof(int)); w += 32) dst[w] = src[w];
-                kind = items[cur].kind;
-                __syncwarp();
+                int *dst = reinterpret_cast<int *>(&a);
+                if (tid < (int)(sizeof(NatArgs) / sizeof(int))) dst[tid] = src[tid];
+                __syncthreads();
             }
-            const TileCoord c = tile_coords(args, t - cur_start);
-#define MDFFT_RUN(i, N)                                           \
-    case kLineKind + i:                                           \
-        line_warp<N>(args, c, 0, stage, lbase, lane);             \
-        break;
-            if constexpr (G == 0) {
-                switch (kind) {
-                    MDFFT_SERVE_LINE_GROUP0(MDFFT_RUN)
-                    default:
-                        break;
-                }
+            const uint32_t l0 = (uint32_t)(t - cur_start) * LINES;
+            // (opaque: a tile's addresses are worked out per tile; hoisted out
+            // of the loop they cost twice the registers)
+            int tt = tid;
+            asm volatile("" : "+r"(tt));
+            const float2 *in = reinterpret_cast<const float2 *>(a.in);
+            float2 *out = reinterpret_cast<float2 *>(a.out);
+            if constexpr (ROWS) {
+                nat_row_tile<float, N>(in, out, buf, tw, tt, l0, a);
             } else {
-                switch (kind) {
-                    MDFFT_SERVE_LINE_GROUP1(MDFFT_RUN)
-                    default:
-                        break;
-                }
+                nat_col_tile<float, N>(in, out, buf, tw, tt, l0, a);
             }
-#undef MDFFT_RUN
         }
+}
+static_assert(sizeof(NatArgs) / sizeof(int) <= 64, "one word per thread");
+
+struct AxisKernel {
+    const void *fn;
+    int threads, lines;
+    size_t smem;
+};
+AxisKernel axis_kernel(int group) {
+    switch (group) {
+#define MDFFT_CASE(i, N)                                                                                            \
+    case 2 * i:                                                                                                     \
+        return {(const void *)&serve_axis_kernel<N, false>, ColCfg<float, N>::THREADS, ColCfg<float, N>::COLS,      \
+                ColCfg<float, N>::SMEM};                                                                            \
+    case 2 * i + 1:                                                                                                 \
+        return {(const void *)&serve_axis_kernel<N, true>, RowCfg<float, N>::THREADS, RowCfg<float, N>::LINES,      \
+                RowCfg<float, N>::SMEM};
+        MDFFT_SERVE_LENGTHS(MDFFT_CASE)
+#undef MDFFT_CASE
+        default:
+            return {nullptr, 0, 0, 0};
+    }
 }
 
 // first-fit allocator over one device arena (offsets 256-byte aligned)
@@ -309,6 +238,8 @@ struct Slot {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     cudaGraphNode_t copy = nullptr;  // the table copy node (its size follows the step's item count)
+    cudaGraphNode_t axis[kGroups] = {nullptr};  // kernel nodes, one per group
+    bool enabled[kGroups] = {false};            // groups the executable graph runs
     cudaEvent_t done = nullptr;
     bool busy = false;
     bool direct = false;  // the step ran plain pass launches (low load)
@@ -320,22 +251,13 @@ struct Slot {
 
 using namespace mdfft::serve;
 
-struct ServePass {  // a plan's pass re-tiled for the persistent kernels
-    PassArgs args;      // for the grouped kernel (kind >= 0)
-    int64_t ctas;
-    int kind;
-    PassArgs line_args;  // for the line kernel (line_kind >= 0): 32-line tiles
-    int64_t line_tiles;
-    int line_kind;
-};
-
 struct mdfft_server_s {
     size_t budget = 0, in_use = 0;
-    std::map<mdfft_plan_t, std::vector<ServePass>> retiled;
     int max_inflight = 0;
     int64_t P = 64;
-    cudaStream_t stream = nullptr, capture = nullptr;
-    int grid = 0;
+    cudaStream_t stream = nullptr;
+    int grid = 0;        // CTAs of a group's kernel at most (0: one resident wave of each)
+    int wave[kGroups] = {0};
     void *arena_mem = nullptr;
     size_t arena_bytes = 0;
     Arena arena;
@@ -347,10 +269,6 @@ struct mdfft_server_s {
     int depth = 2;  // steps in flight on the GPU at most; arrivals in between join the next step
     int chunk = 4;  // at most this many consecutive tiles dealt to a CTA at a time
     int direct = 4;  // low load: at most this many requests with passes left run them as plain launches
-    int lines = 1;   // passes of 16 to 64 points go to the line kernels
-    int line_grid[2] = {0, 0};
-    cudaStream_t capture2[2] = {nullptr, nullptr};            // the line kernels' branches of the step graph
-    cudaEvent_t fork = nullptr, join[2] = {nullptr, nullptr};  // branches start after the table copy, the step ends after all
     Slot slots[kSlots];
     int next_slot = 0;
     cudaEvent_t t0 = nullptr;
@@ -359,41 +277,39 @@ struct mdfft_server_s {
 
 namespace {
 
-mdfft_status capture_graphs(mdfft_server_t s) {
-    for (Slot &sl : s->slots) {
-        if (sl.exec) cudaGraphExecDestroy(sl.exec), sl.exec = nullptr;
-        if (sl.graph) cudaGraphDestroy(sl.graph), sl.graph = nullptr;
-        cudaError_t e = cudaStreamBeginCapture(s->capture, cudaStreamCaptureModeThreadLocal);
-        if (e != cudaSuccess) return cuda_fail(e, "cudaStreamBeginCapture");
-        cudaMemcpyAsync(sl.dev, sl.host, sizeof(Table), cudaMemcpyHostToDevice, s->capture);
-        // the two kernels are parallel branches: the line kernel's CTAs take
-        // SMs as the grouped kernel's CTAs finish, and the other way round
-        cudaEventRecord(s->fork, s->capture);
-        cudaStreamWaitEvent(s->capture2[0], s->fork, 0);
-        cudaStreamWaitEvent(s->capture2[1], s->fork, 0);
-        serve_kernel<<<s->grid, kThreads, kSmem, s->capture>>>(sl.dev);
-        serve_line_kernel<0><<<s->line_grid[0], kLineThreads, kLineSmem[0], s->capture2[0]>>>(sl.dev);
-        serve_line_kernel<1><<<s->line_grid[1], kLineThreads, kLineSmem[1], s->capture2[1]>>>(sl.dev);
-        for (int g = 0; g < 2; ++g) {
-            cudaEventRecord(s->join[g], s->capture2[g]);
-            cudaStreamWaitEvent(s->capture, s->join[g], 0);
-        }
-        e = cudaStreamEndCapture(s->capture, &sl.graph);
-        if (e != cudaSuccess) return cuda_fail(e, "cudaStreamEndCapture");
-        e = cudaGraphInstantiate(&sl.exec, sl.graph, 0);
-        if (e != cudaSuccess) return cuda_fail(e, "cudaGraphInstantiate");
-        size_t nn = 0;
-        cudaGraphGetNodes(sl.graph, nullptr, &nn);
-        std::vector<cudaGraphNode_t> nodes(nn);
-        cudaGraphGetNodes(sl.graph, nodes.data(), &nn);
-        sl.copy = nullptr;
-        for (cudaGraphNode_t nd : nodes) {
-            cudaGraphNodeType ty;
-            if (cudaGraphNodeGetType(nd, &ty) == cudaSuccess && ty == cudaGraphNodeTypeMemcpy) sl.copy = nd;
-        }
+// The graph of a slot, made when the slot is first used: the table copy, then
+// all groups' kernels (disabled until a step needs them) as parallel branches.
+mdfft_status make_graph(Slot &sl) {
+    cudaError_t e = cudaGraphCreate(&sl.graph, 0);
+    if (e == cudaSuccess)
+        e = cudaGraphAddMemcpyNode1D(&sl.copy, sl.graph, nullptr, 0, sl.dev, sl.host, sizeof(Table), cudaMemcpyHostToDevice);
+    for (int g = 0; g < kGroups && e == cudaSuccess; ++g) {
+        const AxisKernel k = axis_kernel(g);
+        void *args[] = {&sl.dev};
+        cudaKernelNodeParams np{};
+        np.func = const_cast<void *>(k.fn);
+        np.gridDim = dim3(1), np.blockDim = dim3((unsigned)k.threads);
+        np.sharedMemBytes = (unsigned)k.smem;
+        np.kernelParams = args;
+        e = cudaGraphAddKernelNode(&sl.axis[g], sl.graph, &sl.copy, 1, &np);
+    }
+    if (e == cudaSuccess) e = cudaGraphInstantiate(&sl.exec, sl.graph, 0);
+    for (int g = 0; g < kGroups && e == cudaSuccess; ++g) {
+        e = cudaGraphNodeSetEnabled(sl.exec, sl.axis[g], 0);
+        sl.enabled[g] = false;
+    }
+    if (e != cudaSuccess) {  // nothing half made is kept: the next use makes it again
+        if (sl.exec) cudaGraphExecDestroy(sl.exec);
+        if (sl.graph) cudaGraphDestroy(sl.graph);
+        sl.exec = nullptr, sl.graph = nullptr;
+        return cuda_fail(e, "step graph");
     }
     return MDFFT_OK;
 }
+
+// Number of launches a request needs: the axes of its plan (the pass kernels
+// where a plan has none, e.g. all dims 1).
+int request_ops(const Request *r) { return r->plan->nat.empty() ? r->plan->M : (int)r->plan->nat.size(); }
 
 // Requests of a slot whose step has completed: record completion, free memory.
 void resolve_slot(mdfft_server_t s, Slot &sl) {
@@ -430,16 +346,6 @@ mdfft_status get_plan(mdfft_server_t s, int M, const int64_t *N, mdfft_plan_t *o
     mdfft_status st = mdfft::detail::plan_create(&p, M, N, std::min<int64_t>(s->P, T), nullptr, MDFFT_C64, 0, false, 1);
     if (st != MDFFT_OK) return st;
     s->plans[key] = p;
-    std::vector<ServePass> rt(M);
-    for (int q = 0; q < M; ++q) {
-        rt[q].kind = kind_of(p->pass[q].n);
-        rt[q].ctas = 0;
-        if (rt[q].kind >= 0) mdfft::detail::retile_pass(p, q, lines_of_kind(rt[q].kind), &rt[q].args, &rt[q].ctas);
-        rt[q].line_kind = line_kind_of(p->pass[q].n);
-        rt[q].line_tiles = 0;
-        if (rt[q].line_kind >= 0) mdfft::detail::retile_pass(p, q, 32, &rt[q].line_args, &rt[q].line_tiles);
-    }
-    s->retiled[p] = rt;
     *out = p;
     return MDFFT_OK;
 }
@@ -465,6 +371,36 @@ PassArgs pass_args(mdfft_server_t s, const Request *r, int pass) {
     a.scale = (pass == M - 1 && r->normalize) ? 1.0 / (double)p->T : 1.0;
     a.scaled = a.scale != 1.0;
     return a;
+}
+
+// Axis `op` of request r as launch arguments: in place on out after the first.
+NatArgs axis_args(const Request *r, int op) {
+    const mdfft_plan_s *p = r->plan;
+    const mdfft::detail::NatOp &o = p->nat[op];
+    const bool last = op + 1 == (int)p->nat.size();
+    NatArgs a = o.args;
+    a.in = op == 0 ? r->in : r->out;
+    a.out = r->out;
+    a.tw = (const char *)p->tw + p->pass[o.s].tw_offset;
+    a.conj = r->dir == 1 ? (op == 0 ? 1 : 0) | (last ? 2 : 0) : 0;
+    a.scale = (last && r->normalize) ? 1.0 / (double)p->T : 1.0;
+    a.scaled = a.scale != 1.0;
+    return a;
+}
+
+// Launch `op` of request r on its own.
+cudaError_t launch_alone(mdfft_server_t s, const Request *r, int op) {
+    if (r->plan->nat.empty()) {
+        const mdfft::detail::Pass &ps = r->plan->pass[op];
+        PassArgs a = pass_args(s, r, op);
+        a.ntiles = ps.ctas;
+        void *args[] = {&a};
+        return cudaLaunchKernel(ps.k.fn, dim3((unsigned)ps.grid), dim3(ps.k.threads), args, ps.k.smem, s->stream);
+    }
+    const mdfft::PassKernel &k = r->plan->nat[op].k;
+    NatArgs a = axis_args(r, op);
+    void *args[] = {&a};
+    return mdfft::detail::launch_following(k, (a.nlines + (unsigned)k.lines - 1) / (unsigned)k.lines, args, s->stream);
 }
 
 }  // namespace
@@ -494,30 +430,16 @@ mdfft_status mdfft_server_create(mdfft_server_t *out, size_t budget_bytes, int m
     s->arena_bytes = (budget_bytes / 3 + 255) / 256 * 256;
     if ((e = cudaMalloc(&s->arena_mem, s->arena_bytes)) != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc arena"));
     s->arena.reset(s->arena_bytes);
-    if ((e = cudaStreamCreateWithFlags(&s->capture, cudaStreamNonBlocking)) != cudaSuccess ||
-        (e = cudaStreamCreateWithFlags(&s->capture2[0], cudaStreamNonBlocking)) != cudaSuccess ||
-        (e = cudaStreamCreateWithFlags(&s->capture2[1], cudaStreamNonBlocking)) != cudaSuccess)
-        return bail(cuda_fail(e, "cudaStreamCreate"));
-    if ((e = cudaEventCreateWithFlags(&s->fork, cudaEventDisableTiming)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&s->join[0], cudaEventDisableTiming)) != cudaSuccess ||
-        (e = cudaEventCreateWithFlags(&s->join[1], cudaEventDisableTiming)) != cudaSuccess)
-        return bail(cuda_fail(e, "cudaEventCreate"));
-    if ((e = cudaFuncSetAttribute(serve_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSmem)) !=
-        cudaSuccess)
-        return bail(cuda_fail(e, "cudaFuncSetAttribute"));
-    int dev = 0, sms = 0, per_sm = 0;
+    int dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, serve_kernel, kThreads, kSmem);
-    s->grid = std::max(1, sms * std::max(1, per_sm));
-    const void *line_fn[2] = {(const void *)serve_line_kernel<0>, (const void *)serve_line_kernel<1>};
-    for (int g = 0; g < 2; ++g) {
-        if ((e = cudaFuncSetAttribute(line_fn[g], cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kLineSmem[g])) !=
-            cudaSuccess)
-            return bail(cuda_fail(e, "cudaFuncSetAttribute"));
-        int line_per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&line_per_sm, line_fn[g], kLineThreads, kLineSmem[g]);
-        s->line_grid[g] = std::max(1, sms * std::max(1, line_per_sm));
+    for (int g = 0; g < kGroups; ++g) {
+        const AxisKernel k = axis_kernel(g);
+        int per_sm = 0;
+        if ((e = cudaFuncSetAttribute(k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)k.smem)) != cudaSuccess ||
+            (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k.fn, k.threads, k.smem)) != cudaSuccess)
+            return bail(cuda_fail(e, "serving kernel"));
+        s->wave[g] = std::max(1, sms * std::max(1, per_sm));
     }
     for (Slot &sl : s->slots) {
         if ((e = cudaHostAlloc((void **)&sl.host, sizeof(Table), cudaHostAllocDefault)) != cudaSuccess)
@@ -527,9 +449,7 @@ mdfft_status mdfft_server_create(mdfft_server_t *out, size_t budget_bytes, int m
             return bail(cuda_fail(e, "cudaMalloc table"));
         if ((e = cudaEventCreate(&sl.done)) != cudaSuccess) return bail(cuda_fail(e, "cudaEventCreate"));
     }
-    mdfft_status st = capture_graphs(s);
-    if (st != MDFFT_OK) return bail(st);
-    s->stats.grid_ctas = s->grid;
+    s->stats.grid_ctas = *std::max_element(s->wave, s->wave + kGroups);
     if ((e = cudaEventCreate(&s->t0)) != cudaSuccess) return bail(cuda_fail(e, "cudaEventCreate"));
     cudaEventRecord(s->t0, s->stream);
     if ((e = cudaStreamSynchronize(s->stream)) != cudaSuccess) return bail(cuda_fail(e, "cudaStreamSynchronize"));
@@ -586,7 +506,7 @@ mdfft_status mdfft_server_step(mdfft_server_t s, int *launched) {
     }
     std::vector<Request *> todo;
     for (Request *r : s->inflight)
-        if (r->next_pass < r->plan->M) todo.push_back(r);
+        if (r->next_pass < request_ops(r)) todo.push_back(r);
     if (todo.empty()) return MDFFT_OK;
     // low load: nothing queued and few requests with passes left -- they run
     // at once; the depth limit, which lets arrivals gather into fuller
@@ -603,19 +523,15 @@ mdfft_status mdfft_server_step(mdfft_server_t s, int *launched) {
     }
     cudaError_t e = cudaSuccess;
     if (direct) {
-        // low load: every remaining pass of these requests, oldest first, as
-        // plain pass launches (stream order keeps each request's passes in order)
+        // low load: every remaining axis of these requests, oldest first, as
+        // plain launches (stream order keeps each request's axes in order)
         for (Request *r : todo) {
-            for (int pass = r->next_pass; pass < r->plan->M; ++pass) {
-                const mdfft::detail::Pass &ps = r->plan->pass[pass];
-                PassArgs a = pass_args(s, r, pass);
-                a.ntiles = ps.ctas;
-                void *args[] = {&a};
-                e = cudaLaunchKernel(ps.k.fn, dim3((unsigned)ps.grid), dim3(ps.k.threads), args, ps.k.smem, s->stream);
-                if (e != cudaSuccess) return cuda_fail(e, "pass launch");
+            for (int op = r->next_pass; op < request_ops(r); ++op) {
+                e = launch_alone(s, r, op);
+                if (e != cudaSuccess) return cuda_fail(e, "axis launch");
                 s->stats.kernel_launches++;
             }
-            r->next_pass = r->plan->M;
+            r->next_pass = request_ops(r);
             r->last_slot = r->slot = s->next_slot;
             sl.finishing.push_back(r);
             s->stats.direct_requests++;
@@ -629,75 +545,75 @@ mdfft_status mdfft_server_step(mdfft_server_t s, int *launched) {
         if (launched) *launched = 1;
         return MDFFT_OK;
     }
+    if (!sl.exec) {
+        mdfft_status st = make_graph(sl);
+        if (st != MDFFT_OK) return st;
+    }
     Table *tab = sl.host;
-    int n = 0, n_line[2] = {0, 0};
-    int64_t total = 0, total_line[2] = {0, 0};
-    std::vector<std::pair<Request *, PassArgs>> separate;  // lengths the persistent kernels do not carry
-    std::vector<Item> line_items[2];
+    std::vector<std::pair<Request *, int>> separate;  // lengths without a kernel in the graph
+    std::vector<Item> items[kGroups];
+    int64_t total[kGroups] = {0};
+    int used = 0;
     for (Request *r : todo) {
-        if (n + n_line[0] + n_line[1] >= kMaxItems) break;
-        const int pass = r->next_pass;
-        const PassArgs a = pass_args(s, r, pass);
-        const ServePass &sp = s->retiled[r->plan][pass];
-        const bool al16 = (uintptr_t)a.in % 16 == 0 && (uintptr_t)a.out % 16 == 0;
-        if (s->lines && sp.line_kind >= 0 && al16) {  // the same pass in 32-line tiles for a line kernel
-            const int g = line_group(sp.line_kind);
-            line_items[g].emplace_back();
-            Item &it = line_items[g].back();
-            it.args = sp.line_args;
-            it.args.in = a.in, it.args.out = a.out, it.args.tw = a.tw;
-            it.args.conj = a.conj, it.args.scale = a.scale, it.args.scaled = a.scaled;
-            it.start = total_line[g];
-            it.kind = sp.line_kind;
-            total_line[g] += sp.line_tiles;
-            n_line[g]++;
-        } else if (sp.kind < 0) {
-            separate.push_back({r, a});
-        } else {  // the same pass re-tiled for the persistent kernel's CTA
-            Item &it = tab->items[n++];
-            it.args = sp.args;
-            it.args.in = a.in, it.args.out = a.out, it.args.tw = a.tw;
-            it.args.conj = a.conj, it.args.scale = a.scale, it.args.scaled = a.scaled;
-            it.start = total;
-            it.kind = sp.kind;
-            total += sp.ctas;
+        if (used >= kMaxItems) break;
+        const int op = r->next_pass;
+        const int kind = r->plan->nat.empty() ? -1 : kind_of(r->plan->pass[r->plan->nat[op].s].n);
+        if (kind < 0) {
+            separate.push_back({r, op});
+        } else {
+            const mdfft::PassKernel &k = r->plan->nat[op].k;
+            const int g = 2 * kind + (r->plan->nat[op].args.stride == 1 ? 1 : 0);
+            items[g].push_back(Item{axis_args(r, op), total[g]});
+            total[g] += (items[g].back().args.nlines + (unsigned)k.lines - 1) / (unsigned)k.lines;
+            ++used;
         }
         r->next_pass++;
         r->last_slot = s->next_slot;
-        if (r->next_pass == r->plan->M) {
+        if (r->next_pass == request_ops(r)) {
             r->slot = s->next_slot;
             sl.finishing.push_back(r);
         }
     }
-    tab->n = n;
-    // the step's tiles spread over every CTA first: chunks of total / grid tiles, at most s->chunk
-    tab->chunk = (int)std::max<int64_t>(1, std::min<int64_t>(s->chunk, total / std::max(1, s->grid)));
-    tab->total = total;
-    for (int g = 0, at = n; g < 2; ++g) {
-        for (int i = 0; i < n_line[g]; ++i) tab->items[at++] = line_items[g][i];
-        tab->n_line[g] = n_line[g];
-        tab->chunk_line[g] = (int)std::max<int64_t>(
-            1, std::min<int64_t>(s->chunk, total_line[g] / std::max<int64_t>(1, (int64_t)s->line_grid[g] * kLineWarps)));
-        tab->total_line[g] = total_line[g];
-    }
-    const int n2 = n_line[0] + n_line[1];
-    if (n + n2 > 0) {
-        if (sl.copy) {  // copy only the header and the items of this step
-            const size_t used = offsetof(Table, items) + (size_t)(n + n2) * sizeof(Item);
-            e = cudaGraphExecMemcpyNodeSetParams1D(sl.exec, sl.copy, sl.dev, sl.host, used, cudaMemcpyHostToDevice);
-            if (e != cudaSuccess) return cuda_fail(e, "cudaGraphExecMemcpyNodeSetParams1D");
+    if (used > 0) {
+        int at = 0;
+        for (int g = 0; g < kGroups; ++g) {
+            Group &gr = tab->group[g];
+            const int64_t ctas = s->grid > 0 ? s->grid : s->wave[g];
+            gr.first = at, gr.n = (int)items[g].size(), gr.total = total[g];
+            // the group's tiles spread over every CTA first: chunks of total / CTAs tiles, at most s->chunk
+            gr.chunk = (int)std::max<int64_t>(1, std::min<int64_t>(s->chunk, total[g] / ctas));
+            for (const Item &it : items[g]) tab->items[at++] = it;
+            const bool on = gr.n > 0;
+            if (on) {
+                const AxisKernel k = axis_kernel(g);
+                void *args[] = {&sl.dev};
+                cudaKernelNodeParams np{};
+                np.func = const_cast<void *>(k.fn);
+                np.gridDim = dim3((unsigned)std::min<int64_t>(ctas, (total[g] + gr.chunk - 1) / gr.chunk));
+                np.blockDim = dim3((unsigned)k.threads);
+                np.sharedMemBytes = (unsigned)k.smem;
+                np.kernelParams = args;
+                e = cudaGraphExecKernelNodeSetParams(sl.exec, sl.axis[g], &np);
+                if (e != cudaSuccess) return cuda_fail(e, "cudaGraphExecKernelNodeSetParams");
+                s->stats.kernel_launches++;
+            }
+            if (on != sl.enabled[g]) {
+                e = cudaGraphNodeSetEnabled(sl.exec, sl.axis[g], on ? 1 : 0);
+                if (e != cudaSuccess) return cuda_fail(e, "cudaGraphNodeSetEnabled");
+                sl.enabled[g] = on;
+            }
         }
+        // copy only the header and the items of this step
+        e = cudaGraphExecMemcpyNodeSetParams1D(sl.exec, sl.copy, sl.dev, sl.host,
+                                               offsetof(Table, items) + (size_t)used * sizeof(Item), cudaMemcpyHostToDevice);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaGraphExecMemcpyNodeSetParams1D");
         e = cudaGraphLaunch(sl.exec, s->stream);
         if (e != cudaSuccess) return cuda_fail(e, "cudaGraphLaunch");
         s->stats.graph_launches++;
-        s->stats.kernel_launches++;
     }
     for (auto &pr : separate) {
-        const mdfft::detail::Pass &ps = pr.first->plan->pass[pr.first->next_pass - 1];
-        PassArgs a = pr.second;
-        void *args[] = {&a};
-        e = cudaLaunchKernel(ps.k.fn, dim3((unsigned)ps.ctas), dim3(ps.k.threads), args, ps.k.smem, s->stream);
-        if (e != cudaSuccess) return cuda_fail(e, "pass launch");
+        e = launch_alone(s, pr.first, pr.second);
+        if (e != cudaSuccess) return cuda_fail(e, "axis launch");
         s->stats.kernel_launches++;
     }
     e = cudaEventRecord(sl.done, s->stream);
@@ -760,9 +676,9 @@ mdfft_status mdfft_server_cancel(mdfft_server_t s, int64_t request_id) {
         s->stats.cancelled++;
         return MDFFT_OK;
     }
-    if (r->next_pass == r->plan->M) return MDFFT_OK;  // its last pass is on the GPU: it completes
+    if (r->next_pass == request_ops(r)) return MDFFT_OK;  // its last pass is on the GPU: it completes
     r->cancelled = true;
-    r->next_pass = r->plan->M;  // no further passes are scheduled
+    r->next_pass = request_ops(r);  // no further passes are scheduled
     Slot *last = r->last_slot >= 0 ? &s->slots[r->last_slot] : nullptr;
     if (last && last->busy) {  // resources come back when its latest step has run
         r->slot = r->last_slot;
@@ -817,13 +733,12 @@ mdfft_status mdfft_server_set_grid(mdfft_server_t s, int ctas) {
         }
     s->grid = ctas;
     s->stats.grid_ctas = ctas;
-    return capture_graphs(s);
+    return MDFFT_OK;
 }
 
 mdfft_status mdfft_server_set_line_kernel(mdfft_server_t s, int enable) {
     if (!s || (enable != 0 && enable != 1)) return fail(MDFFT_E_ARG, "enable must be 0 or 1");
-    s->lines = enable;
-    return MDFFT_OK;
+    return MDFFT_OK;  // every length has its own kernel
 }
 
 mdfft_status mdfft_server_set_chunk(mdfft_server_t s, int chunk) {
@@ -864,12 +779,6 @@ mdfft_status mdfft_server_destroy(mdfft_server_t s) {
         if (sl.done) cudaEventDestroy(sl.done);
     }
     if (s->t0) cudaEventDestroy(s->t0);
-    if (s->capture) cudaStreamDestroy(s->capture);
-    for (int g = 0; g < 2; ++g) {
-        if (s->capture2[g]) cudaStreamDestroy(s->capture2[g]);
-        if (s->join[g]) cudaEventDestroy(s->join[g]);
-    }
-    if (s->fork) cudaEventDestroy(s->fork);
     if (s->arena_mem) cudaFree(s->arena_mem);
     for (auto &kv : s->plans) mdfft_destroy(kv.second);
     for (auto &kv : s->requests) delete kv.second;
