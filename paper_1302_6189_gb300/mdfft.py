@@ -183,13 +183,16 @@ def mdfft_plan_batched(N, P, order=None, dtype=MDFFT_C64, flags=0, batch=1):
 
 
 def mdfft_exec(plan, in_ptr, out_ptr, dir=-1, normalize=0, stream=0):
-    _check(_lib.mdfft_exec(plan, c_void_p(in_ptr), c_void_p(out_ptr), int(dir), int(normalize),
-                           c_void_p(stream)), "mdfft_exec")
+    # (integers go to c_void_p arguments as they are)
+    st = _lib.mdfft_exec(plan, in_ptr, out_ptr, int(dir), int(normalize), stream)
+    if st != MDFFT_OK:
+        raise MdfftError(st, "mdfft_exec")
 
 
 def mdfft_exec_graph(plan, in_ptr, out_ptr, dir=-1, normalize=0, stream=0):
-    _check(_lib.mdfft_exec_graph(plan, c_void_p(in_ptr), c_void_p(out_ptr), int(dir), int(normalize),
-                                 c_void_p(stream)), "mdfft_exec_graph")
+    st = _lib.mdfft_exec_graph(plan, in_ptr, out_ptr, int(dir), int(normalize), stream)
+    if st != MDFFT_OK:
+        raise MdfftError(st, "mdfft_exec_graph")
 
 
 def mdfft_selftest_wait(arrive, limit_us):
@@ -424,7 +427,9 @@ def mdfft_server_poll(server, request_id):
 
 
 def mdfft_server_release(server, request_id):
-    _check(_lib.mdfft_server_release(server, int(request_id)), "mdfft_server_release")
+    st = _lib.mdfft_server_release(server, int(request_id))
+    if st != MDFFT_OK:
+        raise MdfftError(st, "mdfft_server_release")
 
 
 def mdfft_server_cancel(server, request_id):
@@ -475,6 +480,22 @@ def mdfft_last_error():
 
 # ------------------------------------------------------------------- torch convenience
 
+def _raw_stream():
+    """The current stream of the current device as an integer.  Looked up
+    through torch's C functions: torch.cuda.current_stream() builds a Stream
+    object on every call, a good part of a small transform's host time."""
+    global _raw_stream
+    import torch
+    torch.cuda.current_stream()  # initialises CUDA as that call always did
+    device, raw = torch._C._cuda_getDevice, torch._C._cuda_getCurrentRawStream
+
+    def lookup():
+        return raw(device())
+
+    _raw_stream = lookup
+    return lookup()
+
+
 _TORCH_DTYPE = {MDFFT_C64: "complex64", MDFFT_C128: "complex128",
                 MDFFT_C64_TC_FP16: "complex64", MDFFT_C64_TC_BF16: "complex64"}
 
@@ -485,6 +506,7 @@ class Plan:
     independent transforms per execution."""
 
     def __init__(self, shape, P, order=None, dtype="c64", flags=0, batch=1):
+        self._torch_dtype = None  # looked up at the first check
         self.M = len(tuple(shape))
         self.P = int(P)
         self.dtype = DTYPES[dtype] if isinstance(dtype, str) else int(dtype)
@@ -500,20 +522,20 @@ class Plan:
         self.out_shape = out_dims if self.batch == 1 else (self.batch,) + out_dims
 
     def _stream(self, stream):
-        import torch
-        s = torch.cuda.current_stream() if stream is None else stream
-        return s.cuda_stream
+        return _raw_stream() if stream is None else stream.cuda_stream
 
     def _check_tensor(self, t, name, shape=None, cuda=True):
-        import torch
-        want = getattr(torch, _TORCH_DTYPE[self.dtype])
+        want = self._torch_dtype
+        if want is None:
+            import torch
+            want = self._torch_dtype = getattr(torch, _TORCH_DTYPE[self.dtype])
         shape = self.shape if shape is None else shape
-        if not (t.is_cuda == cuda and t.dtype == want and t.is_contiguous() and tuple(t.shape) == shape):
+        if not (t.is_cuda == cuda and t.dtype == want and t.is_contiguous() and t.shape == shape):
             raise ValueError(f"{name} must be a contiguous {'CUDA' if cuda else 'host'} {want} tensor of shape {shape}")
 
     def _out(self, x, out):
-        import torch
         if out is None:
+            import torch
             out = torch.empty(self.out_shape, dtype=x.dtype, device=x.device)
         self._check_tensor(out, "out", self.out_shape)
         return out
@@ -635,16 +657,27 @@ class Server:
         import torch
         s = torch.cuda.current_stream() if stream is None else stream
         self.stream = s
+        self._c64 = torch.complex64
+        self._shape_dims = {}
         self.handle = mdfft_server_create(budget_bytes, max_inflight, P, s.cuda_stream)
 
     def submit(self, x, out, dir=-1, normalize=False):
-        import torch
+        c64 = self._c64
         for t in (x, out):
-            if not (t.is_cuda and t.dtype == torch.complex64 and t.is_contiguous()):
+            if not (t.is_cuda and t.dtype == c64 and t.is_contiguous()):
                 raise ValueError("server requests take contiguous CUDA complex64 tensors")
-        if tuple(x.shape) != tuple(out.shape):
+        shape = x.shape
+        if shape != out.shape:
             raise ValueError("input and output shapes differ")
-        return mdfft_server_submit(self.handle, tuple(x.shape), x.data_ptr(), out.data_ptr(), dir, int(bool(normalize)))
+        dims = self._shape_dims.get(shape)  # one entry per shape, like the server's plans
+        if dims is None:
+            dims = self._shape_dims[shape] = _dims(tuple(shape))[0]
+        rid = i64()
+        st = _lib.mdfft_server_submit(self.handle, len(shape), dims, x.data_ptr(), out.data_ptr(), int(dir),
+                                      int(bool(normalize)), ctypes.byref(rid))
+        if st != MDFFT_OK:
+            raise MdfftError(st, "mdfft_server_submit")
+        return rid.value
 
     def step(self):
         return mdfft_server_step(self.handle)
