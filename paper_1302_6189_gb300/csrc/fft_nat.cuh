@@ -33,6 +33,10 @@
 // 32 4,040 -> 6,020, 96 4,130 -> 5,180, 160 3,940 -> 5,090, 256 5,520 -> 5,960,
 // 512 4,610 -> 5,180; whole transforms: 24^5 170 -> 87 us (64 MB, in L2), 256^3
 // 143 -> 130 us, 512^3 1,190 -> 1,082 us.
+// Double precision: the FP64 units (a warp instruction holds one for 64
+// cycles), so lanes must not idle and small grids need many short-lived warps
+// spread over the SMs: 32^3 25.6 -> 15.9 us, 64^3 44.2 -> 34.5, 128^3 274 -> 256,
+// 48 x 48 planes (2^22 points) 390 -> 317, 256 x 256 399 -> 386.
 #pragma once
 
 #include "nat_args.h"
@@ -103,10 +107,9 @@ template <int N, int F, int C> __host__ __device__ constexpr int digits_out(int 
 // registers) 5,030 / 4,740; 512 = 16 x 16 x 2 5,380 / 6,400, as 16 x 32 4,520 /
 // 5,590; but 480 = 32 x 15 5,090 in columns, as 8 x 4 x 15 4,080.
 __host__ __device__ constexpr int nat_lim(int n, bool dbl, bool rows) {
-    if (dbl) {  // the widest single stage: short chains and many warps for the few FP64 units
-        const int widest = radix_plan(n).maxR;
-        return widest > 8 ? widest : 8;
-    }
+    // double precision: chains as short as the widest stage allows below 60
+    // points, where small grids leave most FP64 units idle
+    if (dbl) return n >= 60 ? 16 : radix_plan(n).maxR > 8 ? radix_plan(n).maxR : 8;
     return n <= 20 ? 20 : n == 480 && !rows ? 32 : 16;
 }
 
@@ -195,9 +198,16 @@ __device__ __forceinline__ double2 ld_cached(const double2 *p) {
 // the next one may be set up while this one runs, and waits here until this
 // one is complete and its stores are visible.  (60 x 240 x 160: 28.7 -> 22.8 us
 // for three launches, 24^5 87.1 -> 77.9 us for five, 256^3 130 -> 122.6 us.)
-__device__ __forceinline__ void follow_previous_launch() {
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+// In single precision the next launch may be set up at once.  In double
+// precision only at a CTA's end: set up early, its CTAs take the places that
+// happen to be free then, and unevenly spread CTAs cost time where FP64 units
+// are the bound (64^3: 87 us against 42 us).
+template <typename Real> __device__ __forceinline__ void follow_previous_launch() {
+    if constexpr (sizeof(Real) == 4) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+template <typename Real> __device__ __forceinline__ void let_next_launch() {
+    if constexpr (sizeof(Real) == 8) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }
 
 template <typename C, int SIZE> __device__ __forceinline__ void conj_all(C (&v)[SIZE]) {
@@ -226,10 +236,27 @@ template <typename Real, int N> struct ColCfg {
     // runs of at least 128 bytes (64-byte runs with half the threads: 384
     // columns 4,890 GB/s against 6,070), and at least 128 threads (96 columns
     // 5,970 GB/s with 128 threads, 5,530 with 256)
-    static constexpr int MINC = 128 / (int)sizeof(C), MINT = 96;
+    static constexpr int MINC = 128 / (int)sizeof(C);
+    // double precision: an FP64 instruction takes a full warp's time whatever
+    // its live lanes, so a warp's 32 / c butterflies of a line have to fit every
+    // part's count up to 1/15 of idle lanes; then the smallest CTA
+    __host__ __device__ static constexpr bool full_warps(int c) {
+        const int w = 32 / c;
+        if (Cfg::TL % w && Cfg::TL != 15) return false;
+        for (int i = 0; i < Cfg::parts.n; ++i) {
+            const int nb = N / Cfg::parts.size[i];
+            if (15 * ((nb + w - 1) / w * w) > 16 * nb) return false;
+        }
+        return true;
+    }
     static constexpr int cols() {
         int c = MINC;
-        while (c * Cfg::TL < MINT && c < 128) c *= 2;
+        if (sizeof(Real) == 8) {
+            while (c < 32 && !full_warps(c) && 2 * c * Cfg::TL <= 512) c *= 2;
+            while (c * Cfg::TL < 32) c *= 2;
+        } else {
+            while (c * Cfg::TL < 96 && c < 128) c *= 2;
+        }
         return c;
     }
     static constexpr int COLS = cols();
@@ -316,7 +343,7 @@ __global__ void __launch_bounds__(ColCfg<Real, N>::THREADS) fft_nat_col_kernel(c
     C *buf = reinterpret_cast<C *>(nat_smem);
     const int tid = threadIdx.x;
     const C *tw = reinterpret_cast<const C *>(a.tw);
-    follow_previous_launch();
+    follow_previous_launch<Real>();
     if constexpr (Cfg::parts.n > 1) {  // twiddles to shared memory; the barrier after the first part covers them
         C *stw = buf + N * CC::COLS;
         for (int q = tid; q < tw_entries(Cfg::plan); q += CC::THREADS) stw[q] = __ldg(tw + q);
@@ -324,6 +351,7 @@ __global__ void __launch_bounds__(ColCfg<Real, N>::THREADS) fft_nat_col_kernel(c
         if constexpr (Cfg::parts.count[0] > 1) __syncthreads();
     }
     nat_col_tile<Real, N>(reinterpret_cast<const C *>(a.in), reinterpret_cast<C *>(a.out), buf, tw, tid, blockIdx.x * CC::COLS, a);
+    let_next_launch<Real>();
 }
 
 // ------------------------------------------------------------------ rows
@@ -342,7 +370,7 @@ __host__ __device__ constexpr NatPad nat_pad(int n, bool dbl, int parts) {
                               {192, 12, 1},  {240, none, 0}, {256, 16, 0}, {320, 20, 1},  {384, 48, 0}, {480, 10, 0},
                               {512, 32, 0},  {640, 40, 8},  {768, 48, 0}, {960, 20, 0},  {1024, 64, 0}};
     constexpr NatPad c128[] = {{10, 5, 1},    {12, none, 0}, {15, none, 0},  {20, 5, 5},   {24, none, 3}, {30, none, 1},
-                               {32, 8, 0},    {40, none, 5}, {48, none, 3},  {60, 5, 1},   {64, 8, 0},    {80, none, 5},
+                               {32, 8, 0},    {40, none, 5}, {48, none, 3},  {60, 64, 0},  {64, 8, 0},    {80, none, 5},
                                {96, 24, 0},   {120, none, 7}, {128, 8, 0},   {160, 40, 0}, {192, 24, 0},  {240, none, 7},
                                {256, 16, 0},  {320, 40, 0},  {384, 24, 0},   {480, 20, 6}, {512, 32, 0},  {640, 40, 0},
                                {768, 48, 0},  {960, 40, 0},  {1024, 64, 0}};
@@ -371,14 +399,22 @@ template <typename Real, int N> struct RowCfg {
     }
     static constexpr bool WARP = even();
     static constexpr int lines() {
-        const int target = sizeof(Real) == 8 ? 32 : Cfg::parts.n == 1 ? 128 : 256;
-        int l = target / Cfg::TL;
-        l = l < 1 ? 1 : l;
-        // double precision: whole warps (an idle lane's share of an FP64 instruction is lost)
-        while (sizeof(Real) == 8 && (l * Cfg::TL) % 32 != 0 && l < 32) ++l;
-        return l;
+        if (sizeof(Real) == 8) {  // full warps in every part (see ColCfg), in a small CTA
+            for (int c = 1; c * Cfg::TL <= 160; ++c) {
+                bool full = c * Cfg::TL > 16 && (Cfg::parts.n > 1 || c % 32 == 0);
+                for (int i = 0; i < Cfg::parts.n; ++i) {
+                    const int items = c * (N / Cfg::parts.size[i]);
+                    full = full && 15 * ((items + 31) / 32 * 32) <= 16 * items;
+                }
+                if (full) return c;
+            }
+            return 160 / Cfg::TL;
+        }
+        const int l = (Cfg::parts.n == 1 ? 128 : 256) / Cfg::TL;
+        return l < 1 ? 1 : l;
     }
-    static constexpr int LINES = lines(), THREADS = LINES * Cfg::TL;
+    static constexpr int LINES = lines();
+    static constexpr int THREADS = sizeof(Real) == 8 ? (LINES * Cfg::TL + 31) / 32 * 32 : LINES * Cfg::TL;
     static_assert(THREADS <= 1024, "CTA shape");
     static constexpr size_t SMEM = (size_t)LINES * RS * sizeof(C);
     // one thread per line of 20 points and more: registers capped for 5 or 6 CTAs per SM
@@ -489,9 +525,10 @@ template <typename Real, int N>
 __global__ void __launch_bounds__(RowCfg<Real, N>::THREADS, RowCfg<Real, N>::MINB) fft_nat_row_kernel(const NatArgs a) {
     using C = typename Cx<Real>::T;
     extern __shared__ __align__(16) unsigned char nat_smem[];
-    follow_previous_launch();
+    follow_previous_launch<Real>();
     nat_row_tile<Real, N>(reinterpret_cast<const C *>(a.in), reinterpret_cast<C *>(a.out), reinterpret_cast<C *>(nat_smem),
                           reinterpret_cast<const C *>(a.tw), threadIdx.x, blockIdx.x * RowCfg<Real, N>::LINES, a);
+    let_next_launch<Real>();
 }
 
 }  // namespace mdfft

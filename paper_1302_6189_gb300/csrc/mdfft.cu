@@ -382,11 +382,11 @@ bool same_plan(const mdfft::RadixPlan &a, const mdfft::RadixPlan &b) {
 
 // The launches of an execution that keeps the natural layout: one per axis
 // longer than 1, in the order of the passes.  None (the pass kernels run) for
-// complex128 and the tensor-core dtypes, spectra left in the last layout, plans that ask
+// the tensor-core dtypes, spectra left in the last layout, plans that ask
 // for the pipelined pass kernels, and arrays of 2^32 lines and more.
 mdfft_status build_nat(mdfft_plan_s *p) {
     p->nat.clear();
-    if (p->dt != MDFFT_C64) return MDFFT_OK;
+    if (p->dt != MDFFT_C64 && p->dt != MDFFT_C128) return MDFFT_OK;
     if (p->flags & (MDFFT_PLAN_OUT_LAST_LAYOUT | MDFFT_PLAN_PERSISTENT)) return MDFFT_OK;
     int64_t stride[pl::kMaxDims], st = 1;
     for (int i = p->M - 1; i >= 0; --i) stride[i] = st, st *= p->N[i];
@@ -397,7 +397,8 @@ mdfft_status build_nat(mdfft_plan_s *p) {
         mdfft::detail::NatOp op;
         op.s = s;
         const bool rows = stride[f] == 1;
-        if (lines + 1024 > 0xffffffffLL || !mdfft::find_nat_kernel_c64(n, rows, &op.k)) {
+        if (lines + 1024 > 0xffffffffLL ||
+            !(p->dt == MDFFT_C64 ? mdfft::find_nat_kernel_c64(n, rows, &op.k) : mdfft::find_nat_kernel_c128(n, rows, &op.k))) {
             p->nat.clear();
             return MDFFT_OK;
         }

@@ -14,17 +14,19 @@ template <typename Real, int N> static PassKernel make_nat(bool rows) {
     return PassKernel{(const void *)&fft_nat_col_kernel<Real, N>, CC::THREADS, CC::COLS, CC::Cfg::TL, CC::SMEM, CC::Cfg::plan};
 }
 
-template <typename Real> static bool find_nat(int64_t n, bool rows, PassKernel *k) {
-    switch (n) {
-#define MDFFT_CASE(N)                       \
-    case N:                                 \
-        *k = make_nat<Real, N>(rows);       \
-        return true;
-        MDFFT_NAT_LENGTHS(MDFFT_CASE)
-#undef MDFFT_CASE
-        default:
-            return false;
+#define MDFFT_FIND_NAT(Real, LENGTHS)              \
+    switch (n) {                                   \
+        LENGTHS(MDFFT_NAT_CASE_##Real)             \
+        default:                                   \
+            return false;                          \
     }
-}
+#define MDFFT_NAT_CASE_float(N) \
+    case N:                     \
+        *k = make_nat<float, N>(rows); \
+        return true;
+#define MDFFT_NAT_CASE_double(N) \
+    case N:                      \
+        *k = make_nat<double, N>(rows); \
+        return true;
 
 }  // namespace mdfft

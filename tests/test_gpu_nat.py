@@ -13,19 +13,21 @@ DEV = torch.device("cuda", 0)
 LENGTHS = [n for n in range(2, 1025) if md.mdfft_supported_length(n, "c64")]
 
 
-def _input(shape, seed):
+def _input(shape, seed, dtype="c64"):
     g = torch.Generator(device=DEV)
     g.manual_seed(seed)
-    return torch.view_as_complex(torch.rand(*shape, 2, generator=g, device=DEV) * 2 - 1)
+    real = torch.float64 if dtype == "c128" else torch.float32
+    return torch.view_as_complex(torch.rand(*shape, 2, generator=g, device=DEV, dtype=real) * 2 - 1)
 
 
+@pytest.mark.parametrize("dtype", ["c64", "c128"])
 @pytest.mark.parametrize("n", LENGTHS)
-def test_every_length_as_rows_and_columns_equals_the_pass_kernels(n):
+def test_every_length_as_rows_and_columns_equals_the_pass_kernels(n, dtype):
     # rows: 3 and 160 lines; columns: 3 and 160 neighbouring lines, one and two blocks of them
     for shape in ((3, n), (n, 3), (160, n), (2, n, 160)):
-        x = _input(shape, n)
+        x = _input(shape, n, dtype)
         keep = x.clone()
-        with md.Plan(shape, 3) as pl:
+        with md.Plan(shape, 3, None, dtype) as pl:
             y = pl.exec(x)
             assert torch.equal(y, pl.exec_counted(x)[0]), shape
             z = pl.exec(x, dir=+1, normalize=True)
