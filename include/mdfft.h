@@ -161,7 +161,10 @@ mdfft_status mdfft_exec(mdfft_plan_t plan, const void *in_dev, void *out_dev, in
                         mdfft_stream_t stream);
 
 /*
- * mdfft_exec_graph -- as mdfft_exec, replayed from a CUDA graph.  The first
+ * mdfft_exec_graph -- as mdfft_exec, with the least launch cost.  A plan whose
+ * execution runs axis launches (see mdfft_launches_per_exec) launches them as
+ * mdfft_exec does: they follow each other without a gap, in less time than a
+ * graph of them.  A plan that runs pass kernels replays a CUDA graph: the first
  * call for a given (in_dev, out_dev, dir, normalize) captures the plan's M
  * pass launches into a graph (on a private stream) and instantiates it; every
  * call then runs the graph with one cudaGraphLaunch on `stream`, which saves
@@ -436,8 +439,9 @@ mdfft_status mdfft_plan_check(mdfft_plan_t plan);
 mdfft_status mdfft_workspace_size(mdfft_plan_t plan, size_t *bytes);
 
 /* Number of kernel launches one mdfft_exec makes: M with the pass kernels,
- * else one per axis longer than 1 (complex64 plans with the default launch
- * choices transform the axes in place, in the natural layout). */
+ * else one per axis longer than 1: complex64 and complex128 plans with the
+ * default launch choices transform the axes in place, in the natural layout
+ * (complex128 unless an axis is 192, 384 or 512). */
 mdfft_status mdfft_launches_per_exec(mdfft_plan_t plan, int *launches);
 
 /* Is line length n built into this library for dtype dt?  1 yes, 0 no. */
