@@ -195,20 +195,14 @@ __device__ __forceinline__ double2 ld_cached(const double2 *p) {
 }
 
 // The launches of an execution follow each other by programmatic dependence:
-// the next one may be set up while this one runs, and waits here until this
-// one is complete and its stores are visible.  (60 x 240 x 160: 28.7 -> 22.8 us
-// for three launches, 24^5 87.1 -> 77.9 us for five, 256^3 130 -> 122.6 us.)
-// In single precision the next launch may be set up at once.  In double
-// precision only at a CTA's end: set up early, its CTAs take the places that
-// happen to be free then, and unevenly spread CTAs cost time where FP64 units
-// are the bound (64^3: 87 us against 42 us).
-template <typename Real> __device__ __forceinline__ void follow_previous_launch() {
-    if constexpr (sizeof(Real) == 4) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-}
-template <typename Real> __device__ __forceinline__ void let_next_launch() {
-    if constexpr (sizeof(Real) == 8) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-}
+// the next one is set up as this one's CTAs leave, and waits here until this
+// one is complete and its stores are visible.  (60 x 240 x 160: 28.7 -> 21.8 us
+// for three launches, 24^5 87.1 -> 75.6 us for five, 256^3 130 -> 121 us.)  The
+// kernels do not let it start any earlier (griddepcontrol.launch_dependents):
+// CTAs set up while others still run take the places that happen to be free,
+// and the uneven spread cost more than the wait saved (80^3 13.4 us against
+// 8.7, 128^3 19.0 / 15.3, 16^5 20.4 / 13.9; complex128 64^3 87 / 34.5).
+__device__ __forceinline__ void follow_previous_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 template <typename C, int SIZE> __device__ __forceinline__ void conj_all(C (&v)[SIZE]) {
 #pragma unroll
@@ -266,7 +260,10 @@ template <typename Real, int N> struct ColCfg {
     static constexpr size_t SMEM = Cfg::parts.n == 1 ? 0 : ((size_t)N * COLS + tw_entries(Cfg::plan)) * sizeof(C);
 };
 
-template <typename Real, int N, int PI> struct ColParts {
+// LOOP: the tile runs in a loop over tiles.  Points of absent lines then get
+// defined values: left alone, their registers would stay live around the loop
+// (and defining them where there is none costs 10 to 50 registers).
+template <typename Real, int N, int PI, bool LOOP> struct ColParts {
     using Cfg = NatCfg<Real, N, false>;
     using C = typename Cfg::C;
     static constexpr int COLS = ColCfg<Real, N>::COLS;
@@ -292,13 +289,13 @@ template <typename Real, int N, int PI> struct ColParts {
 #pragma unroll
                     for (int r = 0; r < SIZE; ++r) v[i][r] = ld_stream(p + (int64_t)(r * D) * a.stride);
                     if (a.conj & 1) conj_all(v[i]);
-                } else {  // (defined values: left alone, they would stay live around a loop over tiles)
+                } else if constexpr (LOOP) {
                     zero_all(v[i]);
                 }
             } else if (live) {
 #pragma unroll
                 for (int r = 0; r < SIZE; ++r) v[i][r] = buf[(at[i] + r * D) * COLS + col];
-            } else {
+            } else if constexpr (LOOP) {
                 zero_all(v[i]);
             }
         }
@@ -319,19 +316,19 @@ template <typename Real, int N, int PI> struct ColParts {
         }
         if constexpr (!LAST) {
             __syncthreads();
-            ColParts<Real, N, PI + 1>::run(src, dst, buf, tw, col, t, ok, a);
+            ColParts<Real, N, PI + 1, LOOP>::run(src, dst, buf, tw, col, t, ok, a);
         }
     }
 };
 
 // Lines l0 .. l0 + COLS - 1 by the whole CTA (tw: the twiddles, staged when the length has an exchange).
-template <typename Real, int N, typename C = typename Cx<Real>::T>
+template <typename Real, int N, bool LOOP = false, typename C = typename Cx<Real>::T>
 __device__ __forceinline__ void nat_col_tile(const C *in, C *out, C *buf, const C *tw, int tid, uint32_t l0, const NatArgs &a) {
     using CC = ColCfg<Real, N>;
     const int col = tid % CC::COLS, t = tid / CC::COLS;
     const uint32_t l = l0 + col, o = fastdiv(l, a.fd);
     const int64_t base = (int64_t)o * N * a.stride + (l - o * a.fd.d);
-    ColParts<Real, N, 0>::run(in + base, out + base, buf, tw, col, t, l < a.nlines, a);
+    ColParts<Real, N, 0, LOOP>::run(in + base, out + base, buf, tw, col, t, l < a.nlines, a);
 }
 
 template <typename Real, int N>
@@ -343,7 +340,7 @@ __global__ void __launch_bounds__(ColCfg<Real, N>::THREADS) fft_nat_col_kernel(c
     C *buf = reinterpret_cast<C *>(nat_smem);
     const int tid = threadIdx.x;
     const C *tw = reinterpret_cast<const C *>(a.tw);
-    follow_previous_launch<Real>();
+    follow_previous_launch();
     if constexpr (Cfg::parts.n > 1) {  // twiddles to shared memory; the barrier after the first part covers them
         C *stw = buf + N * CC::COLS;
         for (int q = tid; q < tw_entries(Cfg::plan); q += CC::THREADS) stw[q] = __ldg(tw + q);
@@ -351,7 +348,6 @@ __global__ void __launch_bounds__(ColCfg<Real, N>::THREADS) fft_nat_col_kernel(c
         if constexpr (Cfg::parts.count[0] > 1) __syncthreads();
     }
     nat_col_tile<Real, N>(reinterpret_cast<const C *>(a.in), reinterpret_cast<C *>(a.out), buf, tw, tid, blockIdx.x * CC::COLS, a);
-    let_next_launch<Real>();
 }
 
 // ------------------------------------------------------------------ rows
@@ -417,12 +413,17 @@ template <typename Real, int N> struct RowCfg {
     static constexpr int THREADS = sizeof(Real) == 8 ? (LINES * Cfg::TL + 31) / 32 * 32 : LINES * Cfg::TL;
     static_assert(THREADS <= 1024, "CTA shape");
     static constexpr size_t SMEM = (size_t)LINES * RS * sizeof(C);
-    // one thread per line of 20 points and more: registers capped for 5 or 6 CTAs per SM
-    static constexpr int MINB = sizeof(Real) == 4 && Cfg::parts.n == 1 && N >= 20 ? (N > 24 ? 5 : 6) : 1;
+    // registers for 40 warps per SM (48 a thread; 32 warps with a 15-point part,
+    // 5 or 6 CTAs with a line of 20 points and more in a thread): uncapped the
+    // compiler spends 60 to 110 on the same code and the warps are missed
+    static constexpr int MINB = sizeof(Real) == 8      ? 1
+                                : Cfg::parts.n == 1    ? (N >= 20 ? 6 : 1)
+                                : Cfg::parts.max == 15 || N % 80 == 0 ? 1024 / THREADS
+                                                       : 1280 / THREADS;
     __host__ __device__ static constexpr int pad(int x) { return x + x / G; }
 };
 
-template <typename Real, int N, int PI> struct RowParts {
+template <typename Real, int N, int PI, bool LOOP> struct RowParts {
     using Cfg = NatCfg<Real, N, true>;
     using RC = RowCfg<Real, N>;
     using C = typename Cfg::C;
@@ -445,7 +446,7 @@ template <typename Real, int N, int PI> struct RowParts {
             k[i] = (int)((unsigned)b % (unsigned)B);
             at[i] = digits_place<N, STAGES>(k[i]) * (N / B) + (int)((unsigned)b / (unsigned)B);
             if (!live[i]) {
-                zero_all(v[i]);
+                if constexpr (LOOP) zero_all(v[i]);
                 continue;
             }
             if constexpr (FIRST) {
@@ -475,13 +476,13 @@ template <typename Real, int N, int PI> struct RowParts {
         if constexpr (!LAST) {
             if constexpr (RC::WARP) __syncwarp();
             else __syncthreads();
-            RowParts<Real, N, PI + 1>::run(in, out, buf, tw, tid, have, a);
+            RowParts<Real, N, PI + 1, LOOP>::run(in, out, buf, tw, tid, have, a);
         }
     }
 };
 
 // Lines l0 .. l0 + LINES - 1 by the whole CTA.
-template <typename Real, int N, typename C = typename Cx<Real>::T>
+template <typename Real, int N, bool LOOP = false, typename C = typename Cx<Real>::T>
 __device__ __forceinline__ void nat_row_tile(const C *in, C *out, C *buf, const C *tw, int tid, uint32_t l0, const NatArgs &a) {
     using RC = RowCfg<Real, N>;
     using Cfg = NatCfg<Real, N, true>;
@@ -517,7 +518,7 @@ __device__ __forceinline__ void nat_row_tile(const C *in, C *out, C *buf, const 
     } else {
         const int64_t base = (int64_t)l0 * N;
         const uint32_t left = a.nlines - l0;
-        RowParts<Real, N, 0>::run(in + base, out + base, buf, tw, tid, left < RC::LINES ? (int)left : RC::LINES, a);
+        RowParts<Real, N, 0, LOOP>::run(in + base, out + base, buf, tw, tid, left < RC::LINES ? (int)left : RC::LINES, a);
     }
 }
 
@@ -525,10 +526,9 @@ template <typename Real, int N>
 __global__ void __launch_bounds__(RowCfg<Real, N>::THREADS, RowCfg<Real, N>::MINB) fft_nat_row_kernel(const NatArgs a) {
     using C = typename Cx<Real>::T;
     extern __shared__ __align__(16) unsigned char nat_smem[];
-    follow_previous_launch<Real>();
+    follow_previous_launch();
     nat_row_tile<Real, N>(reinterpret_cast<const C *>(a.in), reinterpret_cast<C *>(a.out), reinterpret_cast<C *>(nat_smem),
                           reinterpret_cast<const C *>(a.tw), threadIdx.x, blockIdx.x * RowCfg<Real, N>::LINES, a);
-    let_next_launch<Real>();
 }
 
 }  // namespace mdfft

@@ -145,9 +145,9 @@ __global__ void __launch_bounds__(axis_threads<N, ROWS>(), axis_min_ctas<N, ROWS
             const float2 *in = reinterpret_cast<const float2 *>(a.in);
             float2 *out = reinterpret_cast<float2 *>(a.out);
             if constexpr (ROWS) {
-                nat_row_tile<float, N>(in, out, buf, tw, tt, l0, a);
+                nat_row_tile<float, N, true>(in, out, buf, tw, tt, l0, a);
             } else {
-                nat_col_tile<float, N>(in, out, buf, tw, tt, l0, a);
+                nat_col_tile<float, N, true>(in, out, buf, tw, tt, l0, a);
             }
         }
 }
