@@ -182,6 +182,12 @@ __device__ __forceinline__ double2 ld_stream(const double2 *p) {
     return v;
 }
 
+// (written by other SMs in the same launch, fft_pair.cuh: not from L1)
+__device__ __forceinline__ float2 ld_l2(const float2 *p) {
+    float2 v;
+    asm volatile("ld.global.cg.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p) : "memory");
+    return v;
+}
 // (runs shorter than a sector or two: the rest of the sector is read soon, from L1)
 __device__ __forceinline__ float2 ld_cached(const float2 *p) {
     float2 v;
@@ -287,7 +293,10 @@ template <typename Real, int N, int PI, bool LOOP> struct ColParts {
                 if (live && ok) {
                     const C *p = src + (int64_t)at[i] * a.stride;
 #pragma unroll
-                    for (int r = 0; r < SIZE; ++r) v[i][r] = ld_stream(p + (int64_t)(r * D) * a.stride);
+                    for (int r = 0; r < SIZE; ++r) {
+                        if constexpr (LOOP) v[i][r] = ld_l2(p + (int64_t)(r * D) * a.stride);
+                        else v[i][r] = ld_stream(p + (int64_t)(r * D) * a.stride);
+                    }
                     if (a.conj & 1) conj_all(v[i]);
                 } else if constexpr (LOOP) {
                     zero_all(v[i]);

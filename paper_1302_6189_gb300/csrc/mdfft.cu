@@ -415,6 +415,83 @@ mdfft_status build_nat(mdfft_plan_s *p) {
     return MDFFT_OK;
 }
 
+// Which consecutive axes run as one launch (fft_pair.cuh): neighbouring axes of
+// equal length, the first one the inner of a contiguous pair, whole tiles, in
+// arrays larger than L2 keeps between launches (96 MB: 24^5, 64 MB, gains
+// nothing; 256^3, 128 MB, and 64^4 do).
+constexpr int64_t kPairBytes = 96ll << 20;
+mdfft_status build_pairs(mdfft_plan_s *p) {
+    p->pairs.clear();
+    size_t words = 0;
+    if (p->dt != MDFFT_C64 || p->T * p->batch * (int64_t)p->elem < kPairBytes) return MDFFT_OK;
+    for (size_t i = 0; i + 1 < p->nat.size(); ++i) {
+        const mdfft::detail::NatOp &a = p->nat[i], &b = p->nat[i + 1];
+        const int64_t n = p->pass[a.s].n;
+        const bool a_outer = a.args.stride > b.args.stride;
+        const int64_t so = a_outer ? a.args.stride : b.args.stride, si = a_outer ? b.args.stride : a.args.stride;
+        const bool rows = si == 1;
+        if (p->pass[b.s].n != n || so != n * si || (rows && a_outer)) continue;
+        mdfft::detail::PairLaunch pl;
+        int row_tile, col_tile, g;
+        if (!mdfft::find_pair_kernel(n, rows, &pl.k, &row_tile, &col_tile, &g)) continue;
+        if (!rows && si % col_tile) continue;
+        mdfft::PairArgs &q = pl.args;
+        const int64_t unit = n * so, units = p->T * p->batch / unit;  // points that share the coordinates outside
+        int64_t slab_points;
+        for (int o = 0; o < 2; ++o) {
+            q.op[o].io = mdfft::NatArgs{};
+            q.op[o].io.stride = o ? b.args.stride : a.args.stride;
+        }
+        if (rows) {  // slabs of whole planes, at least 512 KB, planes in multiples of the column tiles a CTA takes
+            const int64_t per = std::max<int64_t>(1, (512 << 10) / (unit * (int64_t)p->elem));
+            q.wblocks = 1, q.W = 0;
+            q.units = (uint32_t)units, q.per_slab = (uint32_t)per;
+            q.outer = per * unit;
+            q.slabs = (uint32_t)((units + per - 1) / per);
+            q.op[0].tiles = (uint32_t)(per * n / row_tile), q.op[0].k = 1, q.op[0].step = 0;
+            q.op[1].k = (uint32_t)(n / col_tile), q.op[1].step = unit;
+            q.op[1].tiles = (uint32_t)(per * q.op[1].k / g);
+            slab_points = per * unit;
+            if (q.op[1].k % g) continue;
+        } else {  // blocks of W neighbouring inner points that divide the inner extent, at least 512 KB
+            int64_t k = 1;
+            while (k < si / col_tile && ((si / col_tile) % k || n * n * k * col_tile * (int64_t)p->elem < (512 << 10))) ++k;
+            q.W = (uint32_t)(k * col_tile), q.wblocks = (uint32_t)(si / q.W);
+            q.units = (uint32_t)units, q.per_slab = 1;
+            q.outer = unit;
+            q.slabs = (uint32_t)(units * q.wblocks);
+            for (int o = 0; o < 2; ++o) {
+                q.op[o].k = (uint32_t)k;
+                q.op[o].tiles = (uint32_t)(n * k);
+                q.op[o].step = q.op[o].io.stride == si ? so : si;  // along the other axis
+            }
+            slab_points = n * n * q.W;
+        }
+        int64_t wave = 0;
+        if (pl.k.smem > 48 * 1024) {
+            cudaError_t e = cudaFuncSetAttribute(pl.k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)pl.k.smem);
+            if (e != cudaSuccess) return cuda_fail(e, "cudaFuncSetAttribute");
+        }
+        wave = mdfft::detail::wave_ctas(pl.k);
+        const int64_t total = (int64_t)q.slabs * (q.op[0].tiles + q.op[1].tiles);
+        // 6/5 of the resident CTAs between A's last tile and B's first (256^3 x 8: 64.1 us a volume for the
+        // two axes at 56 slabs of 16 tiles, 65.8 at 32, 76.6 at 96, where L2 no longer holds what is in flight)
+        q.ahead = (uint32_t)std::min<int64_t>(q.slabs, (6 * wave / 5 + q.op[0].tiles - 1) / q.op[0].tiles + 1);
+        if (total + 2 * wave > 0x7fffffffLL || q.ahead * slab_points * (int64_t)p->elem > kPairBytes / 2) continue;
+        pl.op = i;
+        pl.grid = (unsigned)std::min<int64_t>(wave, total);
+        pl.sync = words;
+        words += ((size_t)q.slabs + 3 + 31) / 32 * 32;
+        p->pairs.push_back(pl);
+        ++i;
+    }
+    if (words == 0) return MDFFT_OK;
+    cudaError_t e = cudaMalloc(&p->sync, words * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMemset(p->sync, 0, words * sizeof(uint32_t));
+    if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc counters");
+    return MDFFT_OK;
+}
+
 mdfft_status parse_order(int M, const int *order, std::vector<pl::Layout> &out) {
     out.clear();
     for (int s = 0; s < M; ++s) {
@@ -433,6 +510,7 @@ void release(mdfft_plan_s *p) {
     if (p->tw) cudaFree(p->tw);
     if (p->ws) cudaFree(p->ws);
     if (p->ws2) cudaFree(p->ws2);
+    if (p->sync) cudaFree(p->sync);
     for (cudaEvent_t e : p->ev)
         if (e) cudaEventDestroy(e);
     for (cudaStream_t h : p->hs)
@@ -499,8 +577,32 @@ mdfft_status launch_nat(mdfft_plan_t p, const void *in, void *out, int dir, int 
     const int64_t slot = p->timed % MDFFT_TIMING_SLOTS;
     const size_t ops = p->nat.size();
     int ev = 0;  // events recorded: one before each pass
+    size_t pair = 0;
     for (size_t i = 0; i < ops; ++i) {
         const mdfft::detail::NatOp &op = p->nat[i];
+        if (!one && pair < p->pairs.size() && p->pairs[pair].op == i) {  // ops i and i + 1 (timed as pass i's)
+            const mdfft::detail::PairLaunch &pl = p->pairs[pair++];
+            mdfft::PairArgs g = pl.args;
+            for (int o = 0; o < 2; ++o) {
+                mdfft::NatArgs &q = g.op[o].io;
+                const bool first = i + o == 0, last = i + o + 1 == ops;
+                q.in = (const char *)(first ? in : out) + off;
+                q.out = (char *)out + off;
+                q.conj = dir == 1 ? (first ? 1 : 0) | (last ? 2 : 0) : 0;
+                q.scale = (last && normalize) ? 1.0 / (double)p->T : 1.0;
+                q.scaled = q.scale != 1.0;
+            }
+            g.tw = (const char *)p->tw + p->pass[op.s].tw_offset;
+            g.sync = p->sync + pl.sync;
+            g.err = p->err;
+            if (timed)
+                for (; ev <= op.s; ++ev) cudaEventRecord(p->ev[slot * (p->M + 1) + ev], st);
+            void *args[] = {&g};
+            cudaError_t e = mdfft::detail::launch_following(pl.k, pl.grid, args, st);
+            if (e != cudaSuccess) return cuda_fail(e, "two-axis launch");
+            ++i;
+            continue;
+        }
         mdfft::NatArgs a = op.args;
         if (one) a.nlines = (uint32_t)(a.nlines / p->batch);
         a.in = (const char *)(i == 0 ? in : out) + off;
@@ -803,7 +905,7 @@ mdfft_status mdfft::detail::plan_create(mdfft_plan_t *out, int M, const int64_t 
                     p->pass[s].grid = std::min<int64_t>(p->pass[s].ctas, mdfft::detail::wave_ctas(k));
                 }
             }
-        if ((st = build_nat(p)) != MDFFT_OK) {
+        if ((st = build_nat(p)) != MDFFT_OK || (with_workspace && (st = build_pairs(p)) != MDFFT_OK)) {
             release(p);
             return st;
         }
@@ -1476,7 +1578,7 @@ mdfft_status mdfft_workspace_size(mdfft_plan_t p, size_t *bytes) {
 
 mdfft_status mdfft_launches_per_exec(mdfft_plan_t p, int *launches) {
     if (!p || !launches) return fail(MDFFT_E_ARG, "null argument");
-    *launches = p->as_built && !p->nat.empty() ? (int)p->nat.size() : p->M;
+    *launches = p->as_built && !p->nat.empty() ? (int)(p->nat.size() - p->pairs.size()) : p->M;
     return MDFFT_OK;
 }
 

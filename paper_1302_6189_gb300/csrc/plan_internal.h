@@ -34,6 +34,15 @@ struct NatOp {
     NatArgs args{};      // everything but in/out/tw/conj/scale
 };
 
+// Launches op and op + 1 of NatOp as one (fft_pair.cuh).
+struct PairLaunch {
+    size_t op = 0;
+    PassKernel k{};
+    PairArgs args{};  // everything but in/out/tw/conj/scale/sync/err
+    unsigned grid = 0;
+    size_t sync = 0;  // word offset of its counters in the plan's
+};
+
 // CTAs of one wave of kernel k on the current device (at least 1).
 int64_t wave_ctas(const PassKernel &k);
 
@@ -76,6 +85,8 @@ struct mdfft_plan_s {
     // Launches of an execution that keeps the natural layout; they run while
     // the passes are as built (an autotuned or stored tuning names pass kernels).
     std::vector<mdfft::detail::NatOp> nat;
+    std::vector<mdfft::detail::PairLaunch> pairs;
+    uint32_t *sync = nullptr;  // counters of the two-axis launches (zero between launches)
     std::vector<mdfft::detail::Pass> built;  // the passes as built
     bool as_built = true;
     void *tw = nullptr, *ws = nullptr, *ws2 = nullptr;

@@ -69,3 +69,26 @@ def test_eight_byte_aligned_arrays_and_per_pass_times():
             pl.exec(x, y)
         ms, n = pl.pass_times()
         assert n == 3 and all(t > 0 for t in ms)
+
+
+# arrays of 96 MB and more: neighbouring axes of 64, 128 or 256 points run two to a launch
+@pytest.mark.parametrize("shape,order,batch", [((5, 64, 64), None, 631),                  # whole planes, a ragged last slab
+                                               ((64, 64, 1024), None, 3),                 # blocks of inner points
+                                               ((64, 64, 48), "abc->acb->bca", 64),       # three blocks of 16
+                                               ((64, 64, 48), "abc->bca->acb", 64),       # the outer axis first
+                                               ((64, 64, 64, 64), None, 1),               # two launches for four axes
+                                               ((128, 128, 128), None, 7), ((128, 128, 32), "abc->bca->acb", 24),
+                                               ((3, 256, 256), None, 65), ((256, 256, 16), None, 13)])
+def test_two_axes_in_one_launch_equal_the_pass_kernels(shape, order, batch):
+    full = shape if batch == 1 else (batch,) + shape
+    x = _input(full, 21)
+    with md.Plan(shape, 16, order, batch=batch) as pl:
+        assert pl.launches() < len(shape)
+        want, want_inv = pl.exec_counted(x)[0], pl.exec_counted(x, dir=+1, normalize=True)[0]
+        for _ in range(3):  # the counters of one launch are zero again for the next
+            assert torch.equal(pl.exec(x), want)
+        assert torch.equal(pl.exec(x, dir=+1, normalize=True), want_inv)
+        pl.check()
+    with md.Plan(shape, 16, order, flags=md.MDFFT_PLAN_INPLACE, batch=batch) as pl:
+        buf = x.clone()
+        assert torch.equal(pl.exec(buf, buf), want)
