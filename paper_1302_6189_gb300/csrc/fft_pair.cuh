@@ -69,6 +69,11 @@ template <int N, bool ROWS> struct PairCfg {
     static constexpr int BUF = ROWS && RC::LINES * RC::RS > G * N * CC::COLS ? RC::LINES * RC::RS : G * N * CC::COLS;
     static constexpr size_t SMEM = (size_t)(BUF + NTW) * sizeof(float2);
     static constexpr int MINB = 1280 / THREADS;
+    // a ticket's tile is R of these: 128 bytes a thread, as much as leaves the
+    // tiles of all resident CTAs (25 MB) well inside L2; smaller tickets cost
+    // their barriers and fence more often
+    static constexpr int POINTS = ROWS ? RC::LINES * N : N * CC::COLS;
+    static constexpr int R = POINTS >= 16 * THREADS ? 1 : 16 * THREADS / POINTS;
 };
 
 template <int N, bool ROWS>
@@ -116,31 +121,36 @@ __global__ void __launch_bounds__(PairCfg<N, ROWS>::THREADS, PairCfg<N, ROWS>::M
         const int64_t base = (int64_t)u * a.outer + (int64_t)wb * a.W;
         // units (planes) of this slab; slabs of inner blocks hold one unit
         const uint32_t left = a.units - u * a.per_slab, units = left < a.per_slab ? left : a.per_slab;
-        int me = tid;  // (opaque: a tile's addresses are worked out per tile, not kept around the loop)
-        asm volatile("" : "+r"(me));
-        if (ROWS && op == 0) {
-            if (tile * RC::LINES < units * N) {
-                const int64_t at = base + (int64_t)tile * (RC::LINES * N);
-                RowParts<float, N, 0, true>::run(reinterpret_cast<const float2 *>(a.op[0].io.in) + at,
-                                                 reinterpret_cast<float2 *>(a.op[0].io.out) + at, buf, tw, me, RC::LINES, a.op[0].io);
-            }
-        } else {
-            const int sub = PC::G > 1 ? me / CC::THREADS : 0, m = me - sub * CC::THREADS;
-            const int col = m % CC::COLS, th = m / CC::COLS;
-            const PairOp &o = a.op[ROWS ? 1 : 0];  // (columns: lengths and blocks of both operations alike)
-            const uint32_t ct = tile * PC::G + sub, j = ct / o.k;
-            const bool ok = !ROWS || j < units;
-            const int64_t wat = base + (int64_t)(ct - j * o.k) * CC::COLS + col;
-            if (ROWS || op == 1) {
-                const int64_t at = wat + (int64_t)j * a.op[1].step;
-                ColParts<float, N, 0, true>::run(reinterpret_cast<const float2 *>(a.op[1].io.in) + at,
-                                                 reinterpret_cast<float2 *>(a.op[1].io.out) + at, buf + sub * (N * CC::COLS), tw,
-                                                 col, th, ok, a.op[1].io);
+#pragma unroll 1
+        for (int r = 0; r < PC::R; ++r) {
+            if (r > 0) __syncthreads();  // the exchange buffer is free again
+            const uint32_t part = tile * PC::R + r;
+            int me = tid;  // (opaque: a tile's addresses are worked out per tile, not kept around the loop)
+            asm volatile("" : "+r"(me));
+            if (ROWS && op == 0) {
+                if (part * RC::LINES < units * N) {
+                    const int64_t at = base + (int64_t)part * (RC::LINES * N);
+                    RowParts<float, N, 0, true>::run(reinterpret_cast<const float2 *>(a.op[0].io.in) + at,
+                                                     reinterpret_cast<float2 *>(a.op[0].io.out) + at, buf, tw, me, RC::LINES, a.op[0].io);
+                }
             } else {
-                const int64_t at = wat + (int64_t)j * a.op[0].step;
-                ColParts<float, N, 0, true>::run(reinterpret_cast<const float2 *>(a.op[0].io.in) + at,
-                                                 reinterpret_cast<float2 *>(a.op[0].io.out) + at, buf + sub * (N * CC::COLS), tw,
-                                                 col, th, ok, a.op[0].io);
+                const int sub = PC::G > 1 ? me / CC::THREADS : 0, m = me - sub * CC::THREADS;
+                const int col = m % CC::COLS, th = m / CC::COLS;
+                const PairOp &o = a.op[ROWS ? 1 : 0];  // (columns: lengths and blocks of both operations alike)
+                const uint32_t ct = part * PC::G + sub, j = ct / o.k;
+                const bool ok = !ROWS || j < units;
+                const int64_t wat = base + (int64_t)(ct - j * o.k) * CC::COLS + col;
+                if (ROWS || op == 1) {
+                    const int64_t at = wat + (int64_t)j * a.op[1].step;
+                    ColParts<float, N, 0, true>::run(reinterpret_cast<const float2 *>(a.op[1].io.in) + at,
+                                                     reinterpret_cast<float2 *>(a.op[1].io.out) + at, buf + sub * (N * CC::COLS), tw,
+                                                     col, th, ok, a.op[1].io);
+                } else {
+                    const int64_t at = wat + (int64_t)j * a.op[0].step;
+                    ColParts<float, N, 0, true>::run(reinterpret_cast<const float2 *>(a.op[0].io.in) + at,
+                                                     reinterpret_cast<float2 *>(a.op[0].io.out) + at, buf + sub * (N * CC::COLS), tw,
+                                                     col, th, ok, a.op[0].io);
+                }
             }
         }
         __syncthreads();  // every store of the tile is issued, shared memory is free

@@ -432,8 +432,8 @@ mdfft_status build_pairs(mdfft_plan_s *p) {
         const bool rows = si == 1;
         if (p->pass[b.s].n != n || so != n * si || (rows && a_outer)) continue;
         mdfft::detail::PairLaunch pl;
-        int row_tile, col_tile, g;
-        if (!mdfft::find_pair_kernel(n, rows, &pl.k, &row_tile, &col_tile, &g)) continue;
+        int row_tile, col_tile, g, r;
+        if (!mdfft::find_pair_kernel(n, rows, &pl.k, &row_tile, &col_tile, &g, &r)) continue;
         if (!rows && si % col_tile) continue;
         mdfft::PairArgs &q = pl.args;
         const int64_t unit = n * so, units = p->T * p->batch / unit;  // points that share the coordinates outside
@@ -448,11 +448,11 @@ mdfft_status build_pairs(mdfft_plan_s *p) {
             q.units = (uint32_t)units, q.per_slab = (uint32_t)per;
             q.outer = per * unit;
             q.slabs = (uint32_t)((units + per - 1) / per);
-            q.op[0].tiles = (uint32_t)(per * n / row_tile), q.op[0].k = 1, q.op[0].step = 0;
+            q.op[0].tiles = (uint32_t)(per * n / row_tile / r), q.op[0].k = 1, q.op[0].step = 0;
             q.op[1].k = (uint32_t)(n / col_tile), q.op[1].step = unit;
-            q.op[1].tiles = (uint32_t)(per * q.op[1].k / g);
+            q.op[1].tiles = (uint32_t)(per * q.op[1].k / g / r);
             slab_points = per * unit;
-            if (q.op[1].k % g) continue;
+            if (q.op[1].k % g || (per * n / row_tile) % r || (per * q.op[1].k / g) % r) continue;  // whole tickets
         } else {  // blocks of W neighbouring inner points that divide the inner extent, at least 512 KB
             int64_t k = 1;
             while (k < si / col_tile && ((si / col_tile) % k || n * n * k * col_tile * (int64_t)p->elem < (512 << 10))) ++k;
@@ -462,7 +462,7 @@ mdfft_status build_pairs(mdfft_plan_s *p) {
             q.slabs = (uint32_t)(units * q.wblocks);
             for (int o = 0; o < 2; ++o) {
                 q.op[o].k = (uint32_t)k;
-                q.op[o].tiles = (uint32_t)(n * k);
+                q.op[o].tiles = (uint32_t)(n * k / r);
                 q.op[o].step = q.op[o].io.stride == si ? so : si;  // along the other axis
             }
             slab_points = n * n * q.W;

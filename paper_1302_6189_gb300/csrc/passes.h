@@ -68,8 +68,8 @@ bool find_pass_kernel_line2(int64_t n, int rp, PassKernel *k);  // two threads p
 bool find_nat_kernel_c64(int64_t n, bool rows, PassKernel *k);     // layout kept (fft_nat.cuh): rows or columns
 bool find_nat_kernel_c128(int64_t n, bool rows, PassKernel *k);
 // two neighbouring axes of n points in one launch (fft_pair.cuh), the inner one contiguous (rows) or not:
-// lines of a row tile, columns of a column tile, column tiles per CTA
-bool find_pair_kernel(int64_t n, bool rows, PassKernel *k, int *row_tile, int *col_tile, int *g);
+// lines of a row tile, columns of a column tile, column tiles per CTA, tiles per ticket
+bool find_pair_kernel(int64_t n, bool rows, PassKernel *k, int *row_tile, int *col_tile, int *g, int *r);
 bool find_move_kernel_c64(int64_t n, PassKernel *k);               // data movement of a pass, no FFT
 bool find_move_ring_kernel_c64(int64_t n, int slots, PassKernel *k);  // the same through a ring of slots
 
