@@ -439,7 +439,9 @@ mdfft_status mdfft_plan_check(mdfft_plan_t plan);
 mdfft_status mdfft_workspace_size(mdfft_plan_t plan, size_t *bytes);
 
 /* Number of kernel launches one mdfft_exec makes: M with the pass kernels,
- * else one per axis longer than 1: complex64 and complex128 plans with the
+ * else at most one per axis longer than 1 (neighbouring axes of 64, 128 or 256
+ * points of a complex64 array of 96 MB and more share one), per group of
+ * transforms of a batch that L2 holds (64 MB): complex64 and complex128 plans with the
  * default launch choices transform the axes in place, in the natural layout
  * (complex128 unless an axis is 192, 384 or 512). */
 mdfft_status mdfft_launches_per_exec(mdfft_plan_t plan, int *launches);

@@ -160,8 +160,8 @@ constexpr int kTcSharedBytes = 4112;
 
 // Launch configuration of the pass kernel for line length N.  TC != 0 selects
 // the tensor-core variant (complex64 only): radix-16 stages run as GEMMs.
-// THR != 0 fixes the CTA at THR threads for every length (the persistent
-// serving kernel): a power-of-two number of threads per line and THR / that
+// THR != 0 fixes the CTA at THR threads for every length (tuning variants): a
+// power-of-two number of threads per line and THR / that
 // many lines per tile (stage loops skip butterflies a thread does not own);
 // for a tensor-core kernel THR / (N / 16) lines (one butterfly per thread).
 __host__ __device__ constexpr int pow2ceil(int x) {
@@ -649,9 +649,8 @@ __device__ __forceinline__ void store_tile(const PassArgs &a, const typename Pas
     }
 }
 
-// The whole pass for one tile of lines.  Threads tid >= THREADS (a CTA shared
-// by several line lengths, see the grouped serving kernel) take part in the
-// barriers only.  (Tensor-core plans use the persistent kernel of
+// The whole pass for one tile of lines.  Threads tid >= THREADS take part in
+// the barriers only.  (Tensor-core plans use the persistent kernel of
 // tc_pass.cuh instead.)
 template <typename Real, int N, int TC, int THR = 0, int RP = 0>
 __device__ __forceinline__ void pass_tile(const PassArgs &a, int64_t t, unsigned char *smem_raw, const int tid) {

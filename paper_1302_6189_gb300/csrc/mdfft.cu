@@ -415,15 +415,28 @@ mdfft_status build_nat(mdfft_plan_s *p) {
     return MDFFT_OK;
 }
 
+constexpr int64_t kPairBytes = 96ll << 20;  // more than L2 keeps between launches
+// Transforms of a batch that run through all their axes before the next ones
+// start: as many as L2 keeps between the launches, where the whole batch is
+// more (the batch axis by axis / in groups, us: 24^5 x 4 386 / 305, 20^4 x 100
+// 168 / 125, 128^3 x 8 120 / 103, 64^3 x 256 418 / 392, 30 x 20 x 15 x 2000
+// 142 / 122).  Larger transforms gain nothing: the whole batch runs axis by
+// axis, with the larger launches.
+constexpr int64_t kGroupBytes = 64ll << 20;
+int64_t nat_group(const mdfft_plan_s *p) {
+    const int64_t bytes = p->T * (int64_t)p->elem;
+    if (p->dt != MDFFT_C64 || bytes > kGroupBytes || bytes * p->batch < kPairBytes) return p->batch;
+    return kGroupBytes / bytes;
+}
+
 // Which consecutive axes run as one launch (fft_pair.cuh): neighbouring axes of
 // equal length, the first one the inner of a contiguous pair, whole tiles, in
 // arrays larger than L2 keeps between launches (96 MB: 24^5, 64 MB, gains
 // nothing; 256^3, 128 MB, and 64^4 do).
-constexpr int64_t kPairBytes = 96ll << 20;
 mdfft_status build_pairs(mdfft_plan_s *p) {
     p->pairs.clear();
     size_t words = 0;
-    if (p->dt != MDFFT_C64 || p->T * p->batch * (int64_t)p->elem < kPairBytes) return MDFFT_OK;
+    if (p->dt != MDFFT_C64 || p->T * p->batch * (int64_t)p->elem < kPairBytes || nat_group(p) < p->batch) return MDFFT_OK;
     for (size_t i = 0; i + 1 < p->nat.size(); ++i) {
         const mdfft::detail::NatOp &a = p->nat[i], &b = p->nat[i + 1];
         const int64_t n = p->pass[a.s].n;
@@ -570,8 +583,17 @@ mdfft_status exec_impl(mdfft_plan_t p, const void *in, void *out, int dir, int n
 
 // An execution that keeps the natural layout (no workspace): the first launch
 // reads `in`, the others work in place on `out`.
+// v: the batch (< 0), or nv transforms from v on.
 mdfft_status launch_nat(mdfft_plan_t p, const void *in, void *out, int dir, int normalize, cudaStream_t st, int64_t v,
-                        bool timed) {
+                        bool timed, int64_t nv = 1) {
+    const int64_t group = nat_group(p);
+    if (v < 0 && !timed && group < p->batch) {
+        for (int64_t g = 0; g < p->batch; g += group) {
+            mdfft_status r = launch_nat(p, in, out, dir, normalize, st, g, false, std::min(group, p->batch - g));
+            if (r != MDFFT_OK) return r;
+        }
+        return MDFFT_OK;
+    }
     const bool one = v >= 0 && p->batch > 1;
     const size_t off = v >= 0 ? (size_t)v * (size_t)p->T * p->elem : 0;
     const int64_t slot = p->timed % MDFFT_TIMING_SLOTS;
@@ -604,7 +626,7 @@ mdfft_status launch_nat(mdfft_plan_t p, const void *in, void *out, int dir, int 
             continue;
         }
         mdfft::NatArgs a = op.args;
-        if (one) a.nlines = (uint32_t)(a.nlines / p->batch);
+        if (one) a.nlines = (uint32_t)(a.nlines / p->batch * nv);
         a.in = (const char *)(i == 0 ? in : out) + off;
         a.out = (char *)out + off;
         a.tw = (const char *)p->tw + p->pass[op.s].tw_offset;
@@ -1138,6 +1160,11 @@ mdfft_status mdfft_pass_times(mdfft_plan_t p, float *ms_out, int cap, int *n_exe
             if (e != cudaSuccess) return cuda_fail(e, "cudaEventElapsedTime");
             sum[s] += ms;
         }
+    if (p->as_built)  // two axes of one launch share its time
+        for (const auto &pl : p->pairs) {
+            double &a = sum[p->nat[pl.op].s], &b = sum[p->nat[pl.op + 1].s];
+            a = b = 0.5 * (a + b);
+        }
     for (int s = 0; s < M && s < cap; ++s) ms_out[s] = (float)(sum[s] / (double)n);
     if (n_execs) *n_execs = (int)n;
     return MDFFT_OK;
@@ -1578,7 +1605,8 @@ mdfft_status mdfft_workspace_size(mdfft_plan_t p, size_t *bytes) {
 
 mdfft_status mdfft_launches_per_exec(mdfft_plan_t p, int *launches) {
     if (!p || !launches) return fail(MDFFT_E_ARG, "null argument");
-    *launches = p->as_built && !p->nat.empty() ? (int)(p->nat.size() - p->pairs.size()) : p->M;
+    const int64_t groups = p->nat.empty() ? 1 : (p->batch + nat_group(p) - 1) / nat_group(p);
+    *launches = p->as_built && !p->nat.empty() ? (int)(groups * (int64_t)(p->nat.size() - p->pairs.size())) : p->M;
     return MDFFT_OK;
 }
 

@@ -72,13 +72,13 @@ def test_eight_byte_aligned_arrays_and_per_pass_times():
 
 
 # arrays of 96 MB and more: neighbouring axes of 64, 128 or 256 points run two to a launch
-@pytest.mark.parametrize("shape,order,batch", [((5, 64, 64), None, 631),                  # whole planes, a ragged last slab
-                                               ((64, 64, 1024), None, 3),                 # blocks of inner points
-                                               ((64, 64, 48), "abc->acb->bca", 64),       # three blocks of 16
-                                               ((64, 64, 48), "abc->bca->acb", 64),       # the outer axis first
+@pytest.mark.parametrize("shape,order,batch", [((15, 15, 15, 64, 64), None, 1),           # whole planes, a ragged last slab
+                                               ((64, 64, 5, 640), None, 1),               # blocks of inner points
+                                               ((64, 64, 60, 60), "abcd->abdc->acdb->bcda", 1),
+                                               ((64, 64, 60, 60), "abcd->abdc->bcda->acdb", 1),  # the outer axis first
                                                ((64, 64, 64, 64), None, 1),               # two launches for four axes
-                                               ((128, 128, 128), None, 7), ((128, 128, 32), "abc->bca->acb", 24),
-                                               ((3, 256, 256), None, 65), ((256, 256, 16), None, 13)])
+                                               ((8, 128, 128, 128), None, 1), ((128, 128, 32, 24), "abcd->abdc->bcda->acdb", 1),
+                                               ((192, 256, 256), None, 2), ((256, 256, 240), None, 1)])
 def test_two_axes_in_one_launch_equal_the_pass_kernels(shape, order, batch):
     full = shape if batch == 1 else (batch,) + shape
     x = _input(full, 21)
@@ -92,3 +92,33 @@ def test_two_axes_in_one_launch_equal_the_pass_kernels(shape, order, batch):
     with md.Plan(shape, 16, order, flags=md.MDFFT_PLAN_INPLACE, batch=batch) as pl:
         buf = x.clone()
         assert torch.equal(pl.exec(buf, buf), want)
+
+
+@pytest.mark.parametrize("shape", [(24, 40, 32), (64, 64, 64, 64)])  # axis launches; two-axis launches
+def test_captured_by_the_callers_graph(shape):
+    x, y = _input(shape, 31), None
+    with md.Plan(shape, 16) as pl:
+        want = pl.exec(x).clone()
+        y = torch.empty_like(x)
+        pl.exec(x, y)
+        torch.cuda.synchronize()
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph):
+            pl.exec(x, y)
+        for _ in range(3):
+            y.zero_()
+            graph.replay()
+            assert torch.equal(y, want)
+
+
+@pytest.mark.parametrize("shape,batch", [((24, 24, 24, 24), 41), ((40, 240, 160), 9), ((12, 15, 16), 4400)])
+def test_groups_of_a_batch_equal_the_pass_kernels(shape, batch):
+    # batches of 96 MB and more run in groups of transforms that L2 holds, the last group smaller
+    x = _input((batch,) + shape, 41)
+    with md.Plan(shape, 16, batch=batch) as pl:
+        assert pl.launches() > len(shape)
+        assert torch.equal(pl.exec(x), pl.exec_counted(x)[0])
+        assert torch.equal(pl.exec(x, dir=+1, normalize=True), pl.exec_counted(x, dir=+1, normalize=True)[0])
+        pl.set_timing(True)
+        pl.exec(x)
+        assert len(pl.pass_times()[0]) == len(shape)
