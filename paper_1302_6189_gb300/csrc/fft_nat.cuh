@@ -31,8 +31,8 @@
 // per launch over 2^25 points, GB/s, the pass kernel before (row and column
 // launches together: N x N planes), rows and columns now: N = 24 3,000 -> 6,070,
 // 32 4,040 -> 6,020, 96 4,130 -> 5,180, 160 3,940 -> 5,090, 256 5,520 -> 5,960,
-// 512 4,610 -> 5,180; whole transforms: 24^5 170 -> 87 us (64 MB, in L2), 256^3
-// 143 -> 130 us, 512^3 1,190 -> 1,082 us.
+// 512 4,610 -> 5,180; whole transforms: 24^5 170 -> 76 us (64 MB, in L2), 256^3
+// 142 -> 121 us (108 with fft_pair.cuh), 512^3 1,190 -> 1,056 us.
 // Double precision: the FP64 units (a warp instruction holds one for 64
 // cycles), so lanes must not idle and small grids need many short-lived warps
 // spread over the SMs: 32^3 25.6 -> 15.9 us, 64^3 44.2 -> 34.5, 128^3 274 -> 256,
