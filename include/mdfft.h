@@ -28,8 +28,9 @@
  *    passed in stays owned by the caller; the plan owns its own device
  *    memory (twiddles, workspace) and frees it in mdfft_destroy().
  *  - A plan may be used from one host thread at a time.  Its executions
- *    share the plan's workspace, so executions of one plan on different
- *    streams must be ordered by the caller (events); on one stream they are.
+ *    share the plan's workspace and the counters of its two-axis launches, so
+ *    executions of one plan on different streams must be ordered by the caller
+ *    (events), those of a captured graph too; on one stream they are.
  */
 #ifndef MDFFT_H
 #define MDFFT_H
@@ -187,6 +188,20 @@ mdfft_status mdfft_exec_graph(mdfft_plan_t plan, const void *in_dev, void *out_d
  * device memory for the status.  (Failure detection without a fault.)
  */
 mdfft_status mdfft_selftest_wait(int arrive, int64_t limit_us, int64_t *waited_us);
+
+/*
+ * mdfft_selftest_pair_wait -- runs the plan's first two-axis launch (see
+ * mdfft_launches_per_exec) from in_dev to out_dev (arrays as for mdfft_exec)
+ * with one tile of its first axis left out, so that the second axis waits for
+ * a count that never comes and gives up after limit_us microseconds
+ * (1 .. 10^7).  Returns what mdfft_plan_check then reports, MDFFT_E_TIMEOUT;
+ * the device, the plan and its counters are as before and the next execution
+ * is complete.  out_dev is scratch.  *waited_us (may be NULL) receives the
+ * host-measured duration.  Synchronises the device.  E_UNSUPPORTED for plans
+ * without such a launch.
+ */
+mdfft_status mdfft_selftest_pair_wait(mdfft_plan_t plan, const void *in_dev, void *out_dev, int64_t limit_us,
+                                      int64_t *waited_us);
 
 /*
  * mdfft_exec_counted -- as mdfft_exec, and every pass also counts on the
@@ -428,11 +443,15 @@ mdfft_status mdfft_movement_probe(mdfft_plan_t plan, int s, int slots, int per_s
 mdfft_status mdfft_fp64_rate_probe(double *out_dev, int ctas, int64_t iters, mdfft_stream_t stream,
                                    double *tflops);
 
-/* Waits for the device and reports whether a pass kernel of this plan gave up
- * a bounded wait since the last check (MDFFT_E_TIMEOUT; the affected output
- * is incomplete).  The kernels that wait on the device are the persistent
- * pipelined kernels that mdfft_plan_autotune may select and the tensor-core
- * kernels of MDFFT_C64_TC_FP16 / _BF16 plans (bulk copies, MMA completion). */
+/* Waits for the device and reports whether a kernel of this plan gave up a
+ * bounded wait (2 s) since the last check (MDFFT_E_TIMEOUT; the affected output
+ * is incomplete, although the execution itself, being asynchronous, returned
+ * MDFFT_OK).  The kernels that wait on the device are the two-axis launches of
+ * complex64 plans as made (96 MB and more with neighbouring axes of 64, 128 or
+ * 256 points, see mdfft_launches_per_exec: the second axis of a slab waits for
+ * its first), the persistent pipelined kernels that mdfft_plan_autotune may
+ * select and the tensor-core kernels of MDFFT_C64_TC_FP16 / _BF16 plans (bulk
+ * copies, MMA completion). */
 mdfft_status mdfft_plan_check(mdfft_plan_t plan);
 
 /* Device workspace the plan owns, in bytes (0 for host-only plans). */

@@ -12,11 +12,13 @@
 // Tiles are dealt by a ticket counter.  Tickets are drawn by running CTAs
 // only, and every tile that a B tile waits for has a lower ticket, so it
 // belongs to a CTA that runs or has finished; A tiles wait for nothing, hence
-// every wait ends.  (Waits are bounded all the same: after kPairWaitNs the
-// kernel sets the plan's error flag and every CTA returns.)  The host chooses
-// D so that the tickets between A's last tile of a slab and B's first cover all
+// every wait ends.  (Waits are bounded all the same: after wait_ns the kernel
+// sets the plan's error flag and every CTA returns.)  The host chooses D so
+// that the tickets between A's last tile of a slab and B's first cover all
 // resident CTAs: B rarely waits.  The last CTA to leave zeroes the counters
-// for the next launch.
+// for the next launch: a CTA counts itself out behind a fence, so that what it
+// added to any counter comes before the zeroes.  (After complete waits the B
+// tiles' acquires order this too; after one that gave up nothing else does.)
 //
 // What bounds it: the shared-memory and load/store pipe of the two axes (27 to
 // 31 us per axis and 2^24 points at 256 points, where a trip through HBM takes
@@ -32,8 +34,6 @@
 #include "ptx_sync.cuh"
 
 namespace mdfft {
-
-constexpr uint64_t kPairWaitNs = 2000000000ull;
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p) {
     uint32_t v;
@@ -101,7 +101,7 @@ __global__ void __launch_bounds__(PairCfg<N, ROWS>::THREADS, PairCfg<N, ROWS>::M
                 if (op == 1 && ld_acquire(a.sync + 3 + slab) < a.op[0].tiles) {
                     const uint64_t t0 = global_timer_ns();
                     while (ld_acquire(a.sync + 3 + slab) < a.op[0].tiles) {
-                        if (global_timer_ns() - t0 > kPairWaitNs) {
+                        if (global_timer_ns() - t0 > a.wait_ns) {
                             atomicExch(a.sync + 2, 1);
                             if (a.err) *a.err = 1;
                         }
@@ -161,9 +161,13 @@ __global__ void __launch_bounds__(PairCfg<N, ROWS>::THREADS, PairCfg<N, ROWS>::M
             red_release(a.sync + 3 + slab, 1);
         }
     }
-    if (tid == 0 && atomicAdd(a.sync + 1, 1) == gridDim.x - 1) {  // last one out
-        for (uint32_t s = 0; s < a.slabs; ++s) a.sync[3 + s] = 0;
-        a.sync[0] = a.sync[1] = a.sync[2] = 0;
+    if (tid == 0) {
+        __threadfence();
+        if (atomicAdd(a.sync + 1, 1) == gridDim.x - 1) {  // last one out
+            __threadfence();
+            for (uint32_t s = 0; s < a.slabs; ++s) a.sync[3 + s] = 0;
+            a.sync[0] = a.sync[1] = a.sync[2] = 0;
+        }
     }
 }
 

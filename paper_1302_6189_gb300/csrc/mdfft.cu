@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <chrono>
 #include <cmath>
 #include <cstdio>
 #include <cstring>
@@ -582,6 +583,29 @@ mdfft_status exec_impl(mdfft_plan_t p, const void *in, void *out, int dir, int n
     return launch_passes(p, in, out, dir, normalize, st, counts, -1);
 }
 
+// A two-axis launch's waits give up after this (they end in microseconds).
+constexpr uint64_t kPairWaitNs = 2000000000ull;
+
+// Arguments of two-axis launch pl (element offset `off` bytes into the arrays).
+mdfft::PairArgs pair_args(const mdfft_plan_s *p, const mdfft::detail::PairLaunch &pl, const void *in, void *out, int dir,
+                          int normalize, size_t off) {
+    mdfft::PairArgs g = pl.args;
+    for (size_t o = 0; o < 2; ++o) {
+        mdfft::NatArgs &q = g.op[o].io;
+        const bool first = pl.op + o == 0, last = pl.op + o + 1 == p->nat.size();
+        q.in = (const char *)(first ? in : out) + off;
+        q.out = (char *)out + off;
+        q.conj = dir == 1 ? (first ? 1 : 0) | (last ? 2 : 0) : 0;
+        q.scale = (last && normalize) ? 1.0 / (double)p->T : 1.0;
+        q.scaled = q.scale != 1.0;
+    }
+    g.tw = (const char *)p->tw + p->pass[p->nat[pl.op].s].tw_offset;
+    g.sync = p->sync + pl.sync;
+    g.err = p->err;
+    g.wait_ns = kPairWaitNs;
+    return g;
+}
+
 // An execution that keeps the natural layout (no workspace): the first launch
 // reads `in`, the others work in place on `out`.
 // v: the batch (< 0), or nv transforms from v on.
@@ -605,19 +629,7 @@ mdfft_status launch_nat(mdfft_plan_t p, const void *in, void *out, int dir, int 
         const mdfft::detail::NatOp &op = p->nat[i];
         if (!one && pair < p->pairs.size() && p->pairs[pair].op == i) {  // ops i and i + 1 (timed as pass i's)
             const mdfft::detail::PairLaunch &pl = p->pairs[pair++];
-            mdfft::PairArgs g = pl.args;
-            for (int o = 0; o < 2; ++o) {
-                mdfft::NatArgs &q = g.op[o].io;
-                const bool first = i + o == 0, last = i + o + 1 == ops;
-                q.in = (const char *)(first ? in : out) + off;
-                q.out = (char *)out + off;
-                q.conj = dir == 1 ? (first ? 1 : 0) | (last ? 2 : 0) : 0;
-                q.scale = (last && normalize) ? 1.0 / (double)p->T : 1.0;
-                q.scaled = q.scale != 1.0;
-            }
-            g.tw = (const char *)p->tw + p->pass[op.s].tw_offset;
-            g.sync = p->sync + pl.sync;
-            g.err = p->err;
+            mdfft::PairArgs g = pair_args(p, pl, in, out, dir, normalize, off);
             if (timed)
                 for (; ev <= op.s; ++ev) cudaEventRecord(p->ev[slot * (p->M + 1) + ev], st);
             void *args[] = {&g};
@@ -1587,13 +1599,38 @@ mdfft_status mdfft_plan_check(mdfft_plan_t p) {
     if (!p) return fail(MDFFT_E_ARG, "null plan");
     if (!p->err) return MDFFT_OK;
     int flag = 0;
-    cudaError_t e = cudaMemcpy(&flag, p->err, sizeof(int), cudaMemcpyDeviceToHost);
+    cudaError_t e = cudaDeviceSynchronize();  // (the copy alone waits for no stream made non-blocking)
+    if (e == cudaSuccess) e = cudaMemcpy(&flag, p->err, sizeof(int), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess) return cuda_fail(e, "reading the device status");
     if (flag) {
         cudaMemset(p->err, 0, sizeof(int));
-        return fail(MDFFT_E_TIMEOUT, "a pass kernel's bounded wait gave up; its output is incomplete");
+        return fail(MDFFT_E_TIMEOUT, "a kernel's bounded wait gave up; its output is incomplete");
     }
     return MDFFT_OK;
+}
+
+mdfft_status mdfft_selftest_pair_wait(mdfft_plan_t p, const void *in, void *out, int64_t limit_us, int64_t *waited_us) {
+    if (limit_us < 1 || limit_us > 10000000) return fail(MDFFT_E_ARG, "limit_us must be in [1, 10^7]");
+    mdfft_status st = check_exec(p, in, out, -1, 0, nullptr);
+    if (st != MDFFT_OK) return st;
+    if (!p->as_built || p->pairs.empty()) return fail(MDFFT_E_UNSUPPORTED, "the plan makes no two-axis launch");
+    const mdfft::detail::PairLaunch &pl = p->pairs[0];
+    mdfft::PairArgs g = pair_args(p, pl, in, out, -1, 0, 0);
+    g.wait_ns = (uint64_t)limit_us * 1000;
+    // the ticket counter starts at 1: no CTA draws the first tile of the first
+    // axis, so its slab's count stays one short
+    cudaError_t e = cudaDeviceSynchronize();  // no execution uses the counters
+    if (e == cudaSuccess) e = cudaMemset(g.sync, 1, 1);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e != cudaSuccess) return cuda_fail(e, "two-axis counters");
+    const auto t0 = std::chrono::steady_clock::now();
+    void *args[] = {&g};
+    e = mdfft::detail::launch_following(pl.k, pl.grid, args, nullptr);
+    if (e != cudaSuccess) return cuda_fail(e, "two-axis launch");
+    st = mdfft_plan_check(p);
+    if (waited_us)
+        *waited_us = std::chrono::duration_cast<std::chrono::microseconds>(std::chrono::steady_clock::now() - t0).count();
+    return st;
 }
 
 mdfft_status mdfft_workspace_size(mdfft_plan_t p, size_t *bytes) {

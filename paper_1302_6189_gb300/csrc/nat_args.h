@@ -37,6 +37,7 @@ struct PairArgs {
     uint32_t units, per_slab;  // planes in all and per slab (blocks: outer indices, 1)
     uint32_t *sync;            // [0] ticket, [1] CTAs done, [2] abort, [3 + s] first operation's tiles done in slab s
     int *err;
+    uint64_t wait_ns;          // a wait that takes longer gives up
 };
 
 }  // namespace mdfft

@@ -64,6 +64,7 @@ SIGNATURES = {
     "mdfft_exec": (c_int, [c_void_p, c_void_p, c_void_p, c_int, c_int, c_void_p]),
     "mdfft_exec_graph": (c_int, [c_void_p, c_void_p, c_void_p, c_int, c_int, c_void_p]),
     "mdfft_selftest_wait": (c_int, [c_int, i64, P_(i64)]),
+    "mdfft_selftest_pair_wait": (c_int, [c_void_p, c_void_p, c_void_p, i64, P_(i64)]),
     "mdfft_plan_tuning": (c_int, [c_void_p, P_(ctypes.c_int32), c_int]),
     "mdfft_plan_set_tuning": (c_int, [c_void_p, P_(ctypes.c_int32), c_int]),
     "mdfft_exec_counted": (c_int, [c_void_p, c_void_p, c_void_p, c_int, c_int, c_void_p, c_void_p]),
@@ -199,6 +200,13 @@ def mdfft_selftest_wait(arrive, limit_us):
     """Returns (status, microseconds waited); status MDFFT_E_TIMEOUT when the wait gave up."""
     waited = i64()
     st = _lib.mdfft_selftest_wait(int(arrive), int(limit_us), ctypes.byref(waited))
+    return st, waited.value
+
+
+def mdfft_selftest_pair_wait(plan, in_ptr, out_ptr, limit_us):
+    """Returns (status, microseconds waited); status MDFFT_E_TIMEOUT when the wait gave up."""
+    waited = i64()
+    st = _lib.mdfft_selftest_pair_wait(plan, c_void_p(in_ptr), c_void_p(out_ptr), int(limit_us), ctypes.byref(waited))
     return st, waited.value
 
 
