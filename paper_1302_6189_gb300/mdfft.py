@@ -184,16 +184,13 @@ def mdfft_plan_batched(N, P, order=None, dtype=MDFFT_C64, flags=0, batch=1):
 
 
 def mdfft_exec(plan, in_ptr, out_ptr, dir=-1, normalize=0, stream=0):
-    # (integers go to c_void_p arguments as they are)
-    st = _lib.mdfft_exec(plan, in_ptr, out_ptr, int(dir), int(normalize), stream)
-    if st != MDFFT_OK:
-        raise MdfftError(st, "mdfft_exec")
+    _check(_lib.mdfft_exec(plan, c_void_p(in_ptr), c_void_p(out_ptr), int(dir), int(normalize),
+                           c_void_p(stream)), "mdfft_exec")
 
 
 def mdfft_exec_graph(plan, in_ptr, out_ptr, dir=-1, normalize=0, stream=0):
-    st = _lib.mdfft_exec_graph(plan, in_ptr, out_ptr, int(dir), int(normalize), stream)
-    if st != MDFFT_OK:
-        raise MdfftError(st, "mdfft_exec_graph")
+    _check(_lib.mdfft_exec_graph(plan, c_void_p(in_ptr), c_void_p(out_ptr), int(dir), int(normalize),
+                                 c_void_p(stream)), "mdfft_exec_graph")
 
 
 def mdfft_selftest_wait(arrive, limit_us):
@@ -552,8 +549,11 @@ class Plan:
         """graph=True replays the passes from a CUDA graph captured for these arrays (mdfft_exec_graph)."""
         self._check_tensor(x, "input")
         out = self._out(x, out)
-        run = mdfft_exec_graph if graph else mdfft_exec
-        run(self.handle, x.data_ptr(), out.data_ptr(), dir, int(bool(normalize)), self._stream(stream))
+        # (tensors' addresses are integers: ctypes takes them without the c_void_p objects that refuse other types)
+        run = _lib.mdfft_exec_graph if graph else _lib.mdfft_exec
+        st = run(self.handle, x.data_ptr(), out.data_ptr(), int(dir), 1 if normalize else 0, self._stream(stream))
+        if st != MDFFT_OK:
+            raise MdfftError(st, "mdfft_exec_graph" if graph else "mdfft_exec")
         return out
 
     def exec_counted(self, x, out=None, dir=-1, normalize=False, stream=None):
