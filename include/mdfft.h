@@ -359,8 +359,12 @@ mdfft_status mdfft_pass_describe(mdfft_plan_t plan, int s, mdfft_pass_info *out)
  * variant, tiling and tile order never change results; a different radix
  * plan changes the rounding only.  in_dev (T elements, only read) and out_dev (T elements,
  * overwritten with scratch) are the caller's; the call synchronises `stream`.
- * ms_before / ms_after (M entries each, may be NULL) receive the mean pass
- * times of the default and of the chosen configuration.
+ * A plan that has axis launches (mdfft_launches_per_exec) then times whole
+ * executions by them and by the chosen passes, and keeps the faster: the axis
+ * launches with the passes as made, or the passes.  ms_before / ms_after (M
+ * entries each, may be NULL) receive the mean pass times of the default and of
+ * the chosen pass configuration; where the axis launches are kept, every entry
+ * of ms_after is their time over M.
  */
 /*
  * mdfft_plan_tuning / mdfft_plan_set_tuning -- a plan's launch choices as 4
@@ -386,11 +390,15 @@ mdfft_status mdfft_pass_describe(mdfft_plan_t plan, int s, mdfft_pass_info *out)
  * with 64-line CTAs (48, 60, 64), 25 the same with the alternative radix
  * plan (32, 64), 26 / 27 two threads per line, the stages in registers and
  * one exchange of values between them (32, 64; default / alternative radix
- * plan);
+ * plan), 28 the default kernel, and the plan runs its passes although it has
+ * axis launches;
  * lines per tile along g; lines per tile along h; tile order 0 or 1, see
  * mdfft_pass_info), e.g. after
  * mdfft_plan_autotune, to store and give back to a plan of the same dims, P,
- * order, dtype, batch and flags.  set_tuning checks every pass (variant built
+ * order, dtype, batch and flags.  With the passes as made and no variant 28 a
+ * plan that has axis launches (mdfft_launches_per_exec) runs those, else its
+ * pass kernels; a tuning reads as 28 in every pass where a plan with axis
+ * launches runs its passes as made.  set_tuning checks every pass (variant built
  * for its length and dtype, tile within the kernel's lines and the pass's
  * extents) before changing any; it drops captured graphs.  Results do not
  * depend on the tuning.  cap / n: 4 M.  Host-only plans: E_ARG.

@@ -665,7 +665,7 @@ mdfft_status launch_nat(mdfft_plan_t p, const void *in, void *out, int dir, int 
 mdfft_status launch_passes(mdfft_plan_t p, const void *in, void *out, int dir, int normalize, cudaStream_t st,
                            int64_t *counts, int64_t v, bool allow_timing) {
     const int M = p->M;
-    if (!counts && p->as_built && !p->nat.empty())
+    if (!counts && p->use_nat && !p->nat.empty())
         return launch_nat(p, in, out, dir, normalize, st, v, p->timing && v < 0 && allow_timing);
     const bool one = v >= 0 && p->batch > 1;
     const size_t off = v >= 0 ? (size_t)v * (size_t)p->T * p->elem : 0;
@@ -777,7 +777,7 @@ mdfft_status exec_graph_impl(mdfft_plan_t p, const void *in, void *out, int dir,
     // The axis launches follow each other without a gap and need no capture:
     // launched as they are they take 17.9 us for a 64^3 round trip, as two
     // graphs 24.2 us (32^3 14.7 / 16.4, 128^3 38.7 / 41.0, 24^5 152.7 / 156.7).
-    if (p->as_built && !p->nat.empty()) return launch_nat(p, in, out, dir, normalize, st, -1, false);
+    if (p->use_nat && !p->nat.empty()) return launch_nat(p, in, out, dir, normalize, st, -1, false);
     mdfft_plan_s::GraphEntry *hit = nullptr;
     for (auto &g : p->graphs)
         if (g.in == in && g.out == out && g.dir == dir && g.normalize == normalize) hit = &g;
@@ -1173,7 +1173,7 @@ mdfft_status mdfft_pass_times(mdfft_plan_t p, float *ms_out, int cap, int *n_exe
             if (e != cudaSuccess) return cuda_fail(e, "cudaEventElapsedTime");
             sum[s] += ms;
         }
-    if (p->as_built)  // two axes of one launch share its time
+    if (p->use_nat)  // two axes of one launch share its time
         for (const auto &pl : p->pairs) {
             double &a = sum[p->nat[pl.op].s], &b = sum[p->nat[pl.op + 1].s];
             a = b = 0.5 * (a + b);
@@ -1243,7 +1243,6 @@ mdfft_status mdfft_plan_autotune(mdfft_plan_t p, const void *in, void *out, int 
     if (cudaEventCreate(&e0) != cudaSuccess || cudaEventCreate(&e1) != cudaSuccess)
         return fail(MDFFT_E_CUDA, "cudaEventCreate");
     mdfft_status result = MDFFT_OK;
-    float tuned_ms = 0.f;
     for (int s = 0; s < p->M && result == MDFFT_OK; ++s) {
         Pass &ps = p->pass[s];
         std::vector<PassKernel> variants{ps.k};
@@ -1342,33 +1341,41 @@ mdfft_status mdfft_plan_autotune(mdfft_plan_t p, const void *in, void *out, int 
         ps = best;
         if (ms_before) ms_before[s] = default_ms;
         if (ms_after) ms_after[s] = best_ms;
-        tuned_ms += best_ms;
     }
-    // the launches that keep the natural layout against the sum of the tuned passes
-    p->as_built = passes_as_built(p);
+    p->use_nat = passes_as_built(p);
     if (result == MDFFT_OK && !p->nat.empty()) {
-        float ms = 0.f;
-        for (int w = 0; w < 2 && result == MDFFT_OK; ++w) {
-            const int n = w == 0 ? 2 : reps;
+        // whole executions, the tuned passes (0) against the axis launches (1):
+        // the better of two rounds each, warmed up (with the twiddle tables of
+        // the tuned passes, which do not matter to the time)
+        float best[2] = {0.f, 0.f};
+        p->use_nat = false;
+        for (int w = 0; w < 6 && result == MDFFT_OK; ++w) {
+            const int route = w % 2, n = w < 2 ? 2 : reps;
             cudaEventRecord(e0, st);
-            for (int r = 0; r < n && result == MDFFT_OK; ++r) result = launch_nat(p, in, out, -1, 0, st, -1, false);
+            for (int r = 0; r < n && result == MDFFT_OK; ++r)
+                result = route ? launch_nat(p, in, out, -1, 0, st, -1, false)
+                               : launch_passes(p, in, out, -1, 0, st, nullptr, -1, false);
             cudaEventRecord(e1, st);
             cudaError_t e = cudaEventSynchronize(e1);
             if (result == MDFFT_OK && e != cudaSuccess) result = cuda_fail(e, "autotune launch");
+            float ms = 0.f;
             if (result == MDFFT_OK) cudaEventElapsedTime(&ms, e0, e1);
             ms /= (float)n;
+            if (w == 2 || w == 3 || (w > 3 && ms < best[route])) best[route] = ms;
         }
-        if (result == MDFFT_OK && (p->as_built || ms < tuned_ms)) {
+        if (result == MDFFT_OK && best[1] < best[0]) {
             for (int s = 0; s < p->M; ++s) {
                 if (!same_plan(p->pass[s].k.plan, p->built[s].k.plan)) make_twiddles(p, s, p->built[s].k.plan, st);
                 p->pass[s] = p->built[s];
-                if (ms_after) ms_after[s] = ms / (float)p->M;
+                if (ms_after) ms_after[s] = best[1] / (float)p->M;
             }
-            p->as_built = true;
+            p->use_nat = true;
         }
     }
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
+    const cudaError_t e = cudaStreamSynchronize(st);  // the chosen twiddle tables ready for any stream
+    if (result == MDFFT_OK && e != cudaSuccess) result = cuda_fail(e, "autotune");
     return result;
 }
 
@@ -1385,16 +1392,19 @@ namespace {
 // kernel with a warp-shuffle exchange between its two stages, 17-22 the
 // ring-of-slots kernel (kRing[variant - 17]: slots, CTAs per SM, radix plan),
 // 23-25 one thread per line with the stages in registers (kLine[variant - 23]),
-// 26 / 27 two threads per line (default / alternative radix plan).
+// 26 / 27 two threads per line (default / alternative radix plan), 28 the
+// default kernel in a plan that runs its passes although it has axis launches.
 constexpr int kLineVariant = 17 + kRingVariants;
 constexpr int kLine2Variant = kLineVariant + kLineVariants;
-constexpr int kTuningVariants = kLine2Variant + 2;
+constexpr int kPassesVariant = kLine2Variant + 2;
+constexpr int kTuningVariants = kPassesVariant + 1;
 bool tuning_kernel(const mdfft_plan_s *p, int s, int variant, PassKernel *k) {
     const int64_t n = p->pass[s].n;
     if (variant >= 17 && variant < kLineVariant) return p->dt == MDFFT_C64 && ring_variant(n, variant - 17, true, k);
     if (variant >= kLineVariant && variant < kLine2Variant)
         return p->dt == MDFFT_C64 && line_variant(n, variant - kLineVariant, true, k);
-    if (variant >= kLine2Variant && variant < kTuningVariants)
+    if (variant == kPassesVariant) return lookup(p->dt, n, k);
+    if (variant >= kLine2Variant && variant < kPassesVariant)
         return p->dt == MDFFT_C64 && mdfft::find_pass_kernel_line2(n, variant - kLine2Variant, k);
     switch (variant) {
         case 16:
@@ -1448,6 +1458,7 @@ mdfft_status mdfft_plan_tuning(mdfft_plan_t p, int32_t *out, int cap) {
             if (tuning_kernel(p, s, v, &k) && k.fn == ps.k.fn && k.per_sm == ps.k.per_sm) variant = v;
         }
         if (variant < 0) return fail(MDFFT_E_CUDA, "internal: unknown pass kernel");
+        if (variant == 0 && !p->use_nat && !p->nat.empty() && passes_as_built(p)) variant = kPassesVariant;
         out[4 * s] = variant, out[4 * s + 1] = ps.args.Bg, out[4 * s + 2] = ps.args.Bh, out[4 * s + 3] = ps.mapping;
     }
     return MDFFT_OK;
@@ -1476,8 +1487,12 @@ mdfft_status mdfft_plan_set_tuning(mdfft_plan_t p, const int32_t *in, int n) {
         if (!same_plan(next[s].k.plan, p->pass[s].k.plan)) make_twiddles(p, s, next[s].k.plan, nullptr);
     cudaError_t e = cudaDeviceSynchronize();  // the new tables ready for any stream
     if (e != cudaSuccess) return cuda_fail(e, "twiddle generation");
-    for (int s = 0; s < p->M; ++s) p->pass[s] = next[s];
-    p->as_built = passes_as_built(p);
+    bool passes = false;
+    for (int s = 0; s < p->M; ++s) {
+        p->pass[s] = next[s];
+        passes = passes || in[4 * s] == kPassesVariant;
+    }
+    p->use_nat = !passes && passes_as_built(p);
     drop_graphs(p);
     return MDFFT_OK;
 }
@@ -1613,7 +1628,7 @@ mdfft_status mdfft_selftest_pair_wait(mdfft_plan_t p, const void *in, void *out,
     if (limit_us < 1 || limit_us > 10000000) return fail(MDFFT_E_ARG, "limit_us must be in [1, 10^7]");
     mdfft_status st = check_exec(p, in, out, -1, 0, nullptr);
     if (st != MDFFT_OK) return st;
-    if (!p->as_built || p->pairs.empty()) return fail(MDFFT_E_UNSUPPORTED, "the plan makes no two-axis launch");
+    if (!p->use_nat || p->pairs.empty()) return fail(MDFFT_E_UNSUPPORTED, "the plan makes no two-axis launch");
     const mdfft::detail::PairLaunch &pl = p->pairs[0];
     mdfft::PairArgs g = pair_args(p, pl, in, out, -1, 0, 0);
     g.wait_ns = (uint64_t)limit_us * 1000;
@@ -1644,7 +1659,7 @@ mdfft_status mdfft_workspace_size(mdfft_plan_t p, size_t *bytes) {
 mdfft_status mdfft_launches_per_exec(mdfft_plan_t p, int *launches) {
     if (!p || !launches) return fail(MDFFT_E_ARG, "null argument");
     const int64_t groups = p->nat.empty() ? 1 : (p->batch + nat_group(p) - 1) / nat_group(p);
-    *launches = p->as_built && !p->nat.empty() ? (int)(groups * (int64_t)(p->nat.size() - p->pairs.size())) : p->M;
+    *launches = p->use_nat && !p->nat.empty() ? (int)(groups * (int64_t)(p->nat.size() - p->pairs.size())) : p->M;
     return MDFFT_OK;
 }
 

@@ -82,13 +82,14 @@ struct mdfft_plan_s {
     size_t elem = 8;
     std::vector<mdfft::planner::Layout> order;
     mdfft::detail::Pass pass[MDFFT_MAX_DIMS];
-    // Launches of an execution that keeps the natural layout; they run while
-    // the passes are as built (an autotuned or stored tuning names pass kernels).
+    // Launches of an execution that keeps the natural layout (none: the pass
+    // kernels run); they run while use_nat is set, which takes passes as built
+    // (their twiddle tables) and no tuning that names the pass kernels.
     std::vector<mdfft::detail::NatOp> nat;
     std::vector<mdfft::detail::PairLaunch> pairs;
     uint32_t *sync = nullptr;  // counters of the two-axis launches (zero between launches)
     std::vector<mdfft::detail::Pass> built;  // the passes as built
-    bool as_built = true;
+    bool use_nat = true;
     void *tw = nullptr, *ws = nullptr, *ws2 = nullptr;
     int *err = nullptr;           // device flag set by a persistent kernel whose bounded wait gave up
     bool external_ws = false;     // made by plan_create(..., with_workspace = false)

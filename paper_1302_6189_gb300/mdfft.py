@@ -209,7 +209,7 @@ def mdfft_selftest_pair_wait(plan, in_ptr, out_ptr, limit_us):
 
 TUNING_VARIANTS = ("default", "thr256", "thr512", "pipe1", "pipe2", "tc128", "thr192", "thr384", "radix_alt", "occ6", "tcg", "tcg_direct", "pf2", "pf4",
                    "pf2_radix_alt", "pf4_radix_alt", "shfl256", "ring2x3", "ring3x2", "ring2x4", "ring2x2",
-                   "ring2x3_radix_alt", "ring3x2_radix_alt", "line", "line2w", "line_radix_alt", "line2t", "line2t_radix_alt")
+                   "ring2x3_radix_alt", "ring3x2_radix_alt", "line", "line2w", "line_radix_alt", "line2t", "line2t_radix_alt", "passes")
 
 
 def mdfft_plan_tuning(plan, M):
@@ -603,8 +603,9 @@ class Plan:
         return out_host
 
     def autotune(self, x, scratch, reps=10, stream=None):
-        """Pick the fastest kernel variant and tile shape per pass; returns
-        (ms per pass before, after).  x is only read; scratch is overwritten."""
+        """Pick the fastest kernel variant and tile shape per pass, and the
+        faster of these passes and the axis launches; returns (ms per pass
+        before, after).  x is only read; scratch is overwritten."""
         self._check_tensor(x, "input")
         self._check_tensor(scratch, "scratch", self.out_shape)
         return mdfft_plan_autotune(self.handle, x.data_ptr(), scratch.data_ptr(), reps, self._stream(stream), self.M)
