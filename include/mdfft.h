@@ -295,6 +295,14 @@ mdfft_status mdfft_order_search(int M, const int64_t N[], int64_t P, int want_wo
  * mdfft_pass_times waits for the recorded executions and writes, for each of
  * the M passes (cap entries at most), the mean duration in milliseconds over
  * them; *n_execs (may be NULL) receives how many executions were averaged.
+ * The events stand between the launches and cost about 4 microseconds each, so
+ * time a whole execution without them.  Where an execution runs axis launches
+ * (mdfft_launches_per_exec), entry s is the axis of pass s; two axes of one
+ * launch get half its time each, an axis of length 1 none.  A batch that
+ * otherwise runs in groups of transforms runs axis by axis over the whole batch
+ * while timing is on: M events, and the same results (24^5 x 4: 305 us in
+ * groups, 386 us axis by axis, and 386 us too in groups with an event before
+ * each of their launches).
  */
 #define MDFFT_TIMING_SLOTS 512
 mdfft_status mdfft_pass_timing(mdfft_plan_t plan, int enable);

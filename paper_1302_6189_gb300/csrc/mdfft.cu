@@ -608,7 +608,9 @@ mdfft::PairArgs pair_args(const mdfft_plan_s *p, const mdfft::detail::PairLaunch
 
 // An execution that keeps the natural layout (no workspace): the first launch
 // reads `in`, the others work in place on `out`.
-// v: the batch (< 0), or nv transforms from v on.
+// v: the batch (< 0), or nv transforms from v on.  Timed executions run axis by
+// axis over the whole batch: with events between the launches the groups gain
+// nothing (24^5 x 4: 386 us either way, 305 in groups without events).
 mdfft_status launch_nat(mdfft_plan_t p, const void *in, void *out, int dir, int normalize, cudaStream_t st, int64_t v,
                         bool timed, int64_t nv = 1) {
     const int64_t group = nat_group(p);
