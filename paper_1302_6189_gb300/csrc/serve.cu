@@ -7,8 +7,8 @@
 // axis.  One step is one launch of a CUDA graph: the copy of the step's work
 // table from pinned host memory, then one kernel per line length and kind
 // (rows or columns, fft_nat.cuh) that has work, as parallel branches, so that
-// the tail of one overlaps the others.  The graph of a table slot is made
-// once; a step enables the kernels it needs and sets their grids.
+// the tail of one overlaps the others.  The graphs of the table slots are made
+// with the server; a step enables the kernels it needs and sets their grids.
 //
 // A kernel per length, and not one persistent kernel with all lengths in a
 // switch: that one ran every length at the registers and the shared memory of
@@ -277,8 +277,8 @@ struct mdfft_server_s {
 
 namespace {
 
-// The graph of a slot, made when the slot is first used: the table copy, then
-// all groups' kernels (disabled until a step needs them) as parallel branches.
+// The graph of a slot: the table copy, then all groups' kernels (disabled until
+// a step needs them) as parallel branches.
 mdfft_status make_graph(Slot &sl) {
     cudaError_t e = cudaGraphCreate(&sl.graph, 0);
     if (e == cudaSuccess)
@@ -298,13 +298,7 @@ mdfft_status make_graph(Slot &sl) {
         e = cudaGraphNodeSetEnabled(sl.exec, sl.axis[g], 0);
         sl.enabled[g] = false;
     }
-    if (e != cudaSuccess) {  // nothing half made is kept: the next use makes it again
-        if (sl.exec) cudaGraphExecDestroy(sl.exec);
-        if (sl.graph) cudaGraphDestroy(sl.graph);
-        sl.exec = nullptr, sl.graph = nullptr;
-        return cuda_fail(e, "step graph");
-    }
-    return MDFFT_OK;
+    return e == cudaSuccess ? MDFFT_OK : cuda_fail(e, "step graph");
 }
 
 // Number of launches a request needs: the axes of its plan (the pass kernels
@@ -448,6 +442,7 @@ mdfft_status mdfft_server_create(mdfft_server_t *out, size_t budget_bytes, int m
         if ((e = cudaMalloc((void **)&sl.dev, sizeof(Table))) != cudaSuccess)
             return bail(cuda_fail(e, "cudaMalloc table"));
         if ((e = cudaEventCreate(&sl.done)) != cudaSuccess) return bail(cuda_fail(e, "cudaEventCreate"));
+        if (mdfft_status st = make_graph(sl)) return bail(st);
     }
     s->stats.grid_ctas = *std::max_element(s->wave, s->wave + kGroups);
     if ((e = cudaEventCreate(&s->t0)) != cudaSuccess) return bail(cuda_fail(e, "cudaEventCreate"));
@@ -544,10 +539,6 @@ mdfft_status mdfft_server_step(mdfft_server_t s, int *launched) {
         s->stats.steps++;
         if (launched) *launched = 1;
         return MDFFT_OK;
-    }
-    if (!sl.exec) {
-        mdfft_status st = make_graph(sl);
-        if (st != MDFFT_OK) return st;
     }
     Table *tab = sl.host;
     std::vector<std::pair<Request *, int>> separate;  // lengths without a kernel in the graph
