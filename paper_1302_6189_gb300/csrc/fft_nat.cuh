@@ -210,9 +210,23 @@ __device__ __forceinline__ double2 ld_cached(const double2 *p) {
 // 8.7, 128^3 19.0 / 15.3, 16^5 20.4 / 13.9; complex128 64^3 87 / 34.5).
 __device__ __forceinline__ void follow_previous_launch() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
-template <typename C, int SIZE> __device__ __forceinline__ void conj_all(C (&v)[SIZE]) {
+// In double precision nothing but the butterflies may issue FP64 instructions:
+// one that is predicated off takes its 64 cycles all the same, and the compiler
+// predicates these short blocks.  So a sign is flipped as an integer, and the
+// scale stands in a loop of no or one turn, which stays a branch.  (48-point
+// columns: 911 FP64 instructions per CTA as predicated blocks, 764 needed.)
+__device__ __forceinline__ double flip_sign(double x, unsigned on) {
+    return __hiloint2double(__double2hiint(x) ^ (int)(on << 31), __double2loint(x));
+}
+// conjugation of the first pass's input
+template <typename C, int SIZE> __device__ __forceinline__ void load_conj(C (&v)[SIZE], const NatArgs &a) {
+    if constexpr (sizeof(v[0].x) == 8) {
 #pragma unroll
-    for (int r = 0; r < SIZE; ++r) v[r].y = -v[r].y;
+        for (int r = 0; r < SIZE; ++r) v[r].y = flip_sign(v[r].y, a.conj & 1);
+    } else if (a.conj & 1) {
+#pragma unroll
+        for (int r = 0; r < SIZE; ++r) v[r].y = -v[r].y;
+    }
 }
 template <typename C, int SIZE> __device__ __forceinline__ void zero_all(C (&v)[SIZE]) {
 #pragma unroll
@@ -221,7 +235,15 @@ template <typename C, int SIZE> __device__ __forceinline__ void zero_all(C (&v)[
 // conjugation and scale of the last pass, as store_tile applies them
 template <typename C, int SIZE> __device__ __forceinline__ void finish_all(C (&v)[SIZE], const NatArgs &a) {
     using Real = decltype(v[0].x);
-    if ((a.conj & 2) || a.scaled) {
+    if constexpr (sizeof(Real) == 8) {
+#pragma unroll
+        for (int r = 0; r < SIZE; ++r) v[r].y = flip_sign(v[r].y, (a.conj >> 1) & 1);
+#pragma unroll 1
+        for (int turn = a.scaled; turn > 0; --turn) {
+#pragma unroll
+            for (int r = 0; r < SIZE; ++r) v[r] = C{v[r].x * a.scale, v[r].y * a.scale};
+        }
+    } else if ((a.conj & 2) || a.scaled) {
         const Real sc = (Real)a.scale, sy = (a.conj & 2) ? -sc : sc;
 #pragma unroll
         for (int r = 0; r < SIZE; ++r) v[r] = C{v[r].x * sc, v[r].y * sy};
@@ -297,7 +319,7 @@ template <typename Real, int N, int PI, bool LOOP> struct ColParts {
                         if constexpr (LOOP) v[i][r] = ld_l2(p + (int64_t)(r * D) * a.stride);
                         else v[i][r] = ld_stream(p + (int64_t)(r * D) * a.stride);
                     }
-                    if (a.conj & 1) conj_all(v[i]);
+                    load_conj(v[i], a);
                 } else if constexpr (LOOP) {
                     zero_all(v[i]);
                 }
@@ -462,7 +484,7 @@ template <typename Real, int N, int PI, bool LOOP> struct RowParts {
                 const C *src = in + line[i] * N + at[i];
 #pragma unroll
                 for (int r = 0; r < SIZE; ++r) v[i][r] = D * (int)sizeof(C) >= 64 ? ld_stream(src + r * D) : ld_cached(src + r * D);
-                if (a.conj & 1) conj_all(v[i]);
+                load_conj(v[i], a);
             } else {
 #pragma unroll
                 for (int r = 0; r < SIZE; ++r) v[i][r] = buf[line[i] * RC::RS + RC::pad(at[i] + r * D)];
@@ -513,7 +535,7 @@ __device__ __forceinline__ void nat_row_tile(const C *in, C *out, C *buf, const 
         C v[N];
 #pragma unroll
         for (int r = 0; r < N; ++r) v[r] = row[r];
-        if (a.conj & 1) conj_all(v);
+        load_conj(v, a);
         PartStages<Real, N, true, 0>::run(v, tw);
         finish_all(v, a);
 #pragma unroll
