@@ -67,24 +67,21 @@ template <int N, int RP = 0, int WARPS = 4> struct LineCfg {
     static constexpr size_t SMEM = (size_t)LINES * RS * sizeof(float2) + (size_t)LINES * sizeof(int64_t);
 };
 
-// One warp's 32 lines of tile c: tile lines w0 .. w0 + 31, lane = line - w0.
-// line_issue copies them into the warp's 32 staging rows (RS elements each;
-// lbase: 32 entries) as one cp.async commit group; line_finish, once that
-// group has landed and the warp has met at __syncwarp, transforms and stores
-// them.  line_issue begins with __syncwarp, so a warp may refill rows it has
-// read before.
+// One warp's 32 lines of tile c: tile lines w0 .. w0 + 31, lane = line - w0;
+// stage: the warp's 32 staging rows (RS elements each), lbase: 32 entries.
 template <int N, int RP = 0>
-__device__ __forceinline__ void line_issue(const PassArgs &a, const TileCoord &c, int w0, float2 *stage,
-                                           int64_t *lbase, int lane) {
+__device__ __forceinline__ void line_warp(const PassArgs &a, const TileCoord &c, int w0, float2 *stage,
+                                          int64_t *lbase, int lane) {
     using LC = LineCfg<N, RP, 1>;
     using C = float2;
     const C *in = reinterpret_cast<const C *>(a.in);
+    C *out = reinterpret_cast<C *>(a.out);
+    const C *gtw = reinterpret_cast<const C *>(a.tw);
     const int line = w0 + lane;
     int bg, bh;
     tile_line(a, line, bg, bh);
     const bool ok = line < a.Bg * a.Bh && c.g0 + bg < a.Ng && c.h0 + bh < a.Nh;
     const int64_t ib = c.in_base + (int64_t)bg * a.in_sg + (int64_t)bh * a.in_sh;
-    __syncwarp();  // earlier reads of these rows and offsets are done
     lbase[lane] = ok ? ib : -1;
     __syncwarp();
     // unit e = lane + 32 i is unit u of line l
@@ -98,20 +95,9 @@ __device__ __forceinline__ void line_issue(const PassArgs &a, const TileCoord &c
         }
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
-}
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    __syncwarp();
 
-template <int N, int RP = 0>
-__device__ __forceinline__ void line_finish(const PassArgs &a, const TileCoord &c, int w0, const float2 *stage,
-                                            int lane) {
-    using LC = LineCfg<N, RP, 1>;
-    using C = float2;
-    C *out = reinterpret_cast<C *>(a.out);
-    const C *gtw = reinterpret_cast<const C *>(a.tw);
-    const int line = w0 + lane;
-    int bg, bh;
-    tile_line(a, line, bg, bh);
-    const bool ok = line < a.Bg * a.Bh && c.g0 + bg < a.Ng && c.h0 + bh < a.Nh;
-    const int64_t ib = c.in_base + (int64_t)bg * a.in_sg + (int64_t)bh * a.in_sh;
     C x[N];
     const C *row = stage + lane * LC::RS;
 #pragma unroll
@@ -155,16 +141,6 @@ __device__ __forceinline__ void line_finish(const PassArgs &a, const TileCoord &
             if (split) atomicAdd(a.split, split);
         }
     }
-}
-
-// The whole tile for one warp: copy, wait, transform and store.
-template <int N, int RP = 0>
-__device__ __forceinline__ void line_warp(const PassArgs &a, const TileCoord &c, int w0, float2 *stage,
-                                          int64_t *lbase, int lane) {
-    line_issue<N, RP>(a, c, w0, stage, lbase, lane);
-    asm volatile("cp.async.wait_group 0;" ::: "memory");
-    __syncwarp();
-    line_finish<N, RP>(a, c, w0, stage, lane);
 }
 
 // One tile of LINES = 32 WARPS lines per CTA; warp w takes tile lines 32 w ..
@@ -214,7 +190,6 @@ __device__ __forceinline__ void line2_warp(const PassArgs &a, const TileCoord &c
     tile_line(a, line, bg, bh);
     const bool ok = line < a.Bg * a.Bh && c.g0 + bg < a.Ng && c.h0 + bh < a.Nh;
     const int64_t ib = c.in_base + (int64_t)bg * a.in_sg + (int64_t)bh * a.in_sh;
-    __syncwarp();  // earlier reads of these rows and offsets are done (a warp may run tile after tile)
     if (t == 0) lbase[l] = ok ? ib : -1;
     __syncwarp();
     // the warp's 16 lines into its rows: unit e = lane + 32 i is unit u of line ll

@@ -580,16 +580,15 @@ __device__ __forceinline__ void store_tile(const PassArgs &a, const typename Pas
     using Cfg = PassCfg<Real, N, TC, THR, RP>;
     using C = typename Cfg::C;
     C *out = reinterpret_cast<C *>(a.out);
-    const bool active = tid < Cfg::THREADS;
     const int sl = tid % Cfg::LINES, k0 = tid / Cfg::LINES;
     int sbg, sbh;
     tile_line(a, sl, sbg, sbh);
-    const bool sok = active && sl < a.Bg * a.Bh && c.g0 + sbg < a.Ng && c.h0 + sbh < a.Nh;
+    const bool sok = sl < a.Bg * a.Bh && c.g0 + sbg < a.Ng && c.h0 + sbh < a.Nh;
     unsigned long long moved = 0, split = 0;
     if (a.line_store) {  // the output keeps f fastest: every line is stored whole, k fastest across lanes
         const bool plain = !(a.conj & 2) && !a.scaled;
         const Real sc = plain ? (Real)1 : (Real)a.scale, sy = (a.conj & 2) ? -sc : sc;
-        for (int e = tid; e < Cfg::LINES * N && active; e += Cfg::THREADS) {
+        for (int e = tid; e < Cfg::LINES * N; e += Cfg::THREADS) {
             const int l = e / N, k = e % N;
             int bg, bh;
             tile_line(a, l, bg, bh);
@@ -649,9 +648,8 @@ __device__ __forceinline__ void store_tile(const PassArgs &a, const typename Pas
     }
 }
 
-// The whole pass for one tile of lines.  Threads tid >= THREADS take part in
-// the barriers only.  (Tensor-core plans use the persistent kernel of
-// tc_pass.cuh instead.)
+// The whole pass for one tile of lines.  (Tensor-core plans use the persistent
+// kernel of tc_pass.cuh instead.)
 template <typename Real, int N, int TC, int THR = 0, int RP = 0>
 __device__ __forceinline__ void pass_tile(const PassArgs &a, int64_t t, unsigned char *smem_raw, const int tid) {
     using Cfg = PassCfg<Real, N, TC, THR, RP>;
@@ -660,8 +658,6 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, int64_t t, unsigned
     C *tw = buf + Cfg::DATA;
     int64_t *lbase = reinterpret_cast<int64_t *>(tw + Cfg::TWN + Cfg::BFRAG);  // input offset of each tile line
     TileCoord *shc = reinterpret_cast<TileCoord *>(lbase + Cfg::LINES);
-    const bool active = tid < Cfg::THREADS;
-
     const C *in = reinterpret_cast<const C *>(a.in);
     const C *gtw = reinterpret_cast<const C *>(a.tw);
 
@@ -676,8 +672,7 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, int64_t t, unsigned
             lbase[l] = w0.in_base + bg * a.in_sg + bh * a.in_sh;
         }
     }
-    if (active)
-        for (int q = tid; q < tw_entries(Cfg::plan); q += Cfg::THREADS) tw[q] = gtw[q];
+    for (int q = tid; q < tw_entries(Cfg::plan); q += Cfg::THREADS) tw[q] = gtw[q];
     __syncthreads();
     const TileCoord c = *shc;
 
@@ -685,32 +680,29 @@ __device__ __forceinline__ void pass_tile(const PassArgs &a, int64_t t, unsigned
     const int line = tid / Cfg::TL, tl = tid % Cfg::TL;
     int fbg, fbh;
     tile_line(a, line, fbg, fbh);
-    const bool fok = active && line < a.Bg * a.Bh && c.g0 + fbg < a.Ng && c.h0 + fbh < a.Nh;
+    const bool fok = line < a.Bg * a.Bh && c.g0 + fbg < a.Ng && c.h0 + fbh < a.Nh;
 
     if constexpr (!Cfg::DIRECT) {  // stage the whole tile through shared memory
-        if (active) {
-            for (int e = tid; e < Cfg::LINES * N; e += Cfg::THREADS) {
-                const int l = e / N, i = e % N;
-                int bg, bh;
-                tile_line(a, l, bg, bh);
-                if (l < a.Bg * a.Bh && c.g0 + bg < a.Ng && c.h0 + bh < a.Nh) {
-                    C x = in[lbase[l] + i];
-                    if (a.conj & 1) x.y = -x.y;
-                    buf[l * Cfg::PADN + padg<Cfg::PADG>(i)] = x;
-                }
+        for (int e = tid; e < Cfg::LINES * N; e += Cfg::THREADS) {
+            const int l = e / N, i = e % N;
+            int bg, bh;
+            tile_line(a, l, bg, bh);
+            if (l < a.Bg * a.Bh && c.g0 + bg < a.Ng && c.h0 + bh < a.Nh) {
+                C x = in[lbase[l] + i];
+                if (a.conj & 1) x.y = -x.y;
+                buf[l * Cfg::PADN + padg<Cfg::PADG>(i)] = x;
             }
         }
         __syncthreads();
     }
     if constexpr (Cfg::plan.S == 0) {  // length-1 lines: the DFT is the identity
-        C v = C{0, 0};
-        if (active) v = buf[line * Cfg::PADN];
+        const C v = buf[line * Cfg::PADN];
         __syncthreads();
-        if (active) buf[line] = v;  // tile[k = 0][line]
+        buf[line] = v;  // tile[k = 0][line]
         __syncthreads();
     } else {
-        const C *gsrc = in + lbase[line < Cfg::LINES ? line : 0];
-        Stages<Real, N, 0, 1, TC, THR, -1, RP>::run(buf, buf, tw, gsrc, line, tl, fok, (a.conj & 1) != 0, active);
+        const C *gsrc = in + lbase[line];
+        Stages<Real, N, 0, 1, TC, THR, -1, RP>::run(buf, buf, tw, gsrc, line, tl, fok, (a.conj & 1) != 0, true);
     }
     store_tile<Real, N, TC, THR, RP>(a, buf, lbase, c, tid);
 }
