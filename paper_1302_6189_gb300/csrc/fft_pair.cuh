@@ -16,8 +16,8 @@
 // sets the plan's error flag and every CTA returns.)  The host chooses D so
 // that the tickets between A's last tile of a slab and B's first cover all
 // resident CTAs: B rarely waits.  The last CTA to leave zeroes the counters
-// for the next launch: a CTA counts itself out behind a fence, so that what it
-// added to any counter comes before the zeroes.  (After complete waits the B
+// for the next launch: a CTA counts itself out with release and acquire, so
+// that what it added to any counter comes before the zeroes.  (After complete waits the B
 // tiles' acquires order this too; after one that gave up nothing else does.)
 //
 // What bounds it: the shared-memory and load/store pipe of the two axes (27 to
@@ -42,6 +42,12 @@ __device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p) {
 }
 __device__ __forceinline__ void red_release(uint32_t *p, uint32_t v) {
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ uint32_t add_acq_rel(uint32_t *p, uint32_t v) {
+    uint32_t old;
+    asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
+    return old;
 }
 
 // ticket -> operation, slab, tile: A of the first D slabs, then per slab i the
@@ -161,13 +167,9 @@ __global__ void __launch_bounds__(PairCfg<N, ROWS>::THREADS, PairCfg<N, ROWS>::M
             red_release(a.sync + 3 + slab, 1);
         }
     }
-    if (tid == 0) {
-        __threadfence();
-        if (atomicAdd(a.sync + 1, 1) == gridDim.x - 1) {  // last one out
-            __threadfence();
-            for (uint32_t s = 0; s < a.slabs; ++s) a.sync[3 + s] = 0;
-            a.sync[0] = a.sync[1] = a.sync[2] = 0;
-        }
+    if (tid == 0 && add_acq_rel(a.sync + 1, 1) == gridDim.x - 1) {  // last one out
+        for (uint32_t s = 0; s < a.slabs; ++s) a.sync[3 + s] = 0;
+        a.sync[0] = a.sync[1] = a.sync[2] = 0;
     }
 }
 
