@@ -213,7 +213,7 @@ __device__ __forceinline__ void follow_previous_launch() { asm volatile("griddep
 // In double precision nothing but the butterflies may issue FP64 instructions:
 // one that is predicated off takes its 64 cycles all the same, and the compiler
 // predicates these short blocks.  So a sign is flipped as an integer, and the
-// scale stands in a loop of no or one turn, which stays a branch.  (48-point
+// scaled stores stand in a block of their own, which stays a branch.  (48-point
 // columns: 911 FP64 instructions per CTA as predicated blocks, 764 needed.)
 __device__ __forceinline__ double flip_sign(double x, unsigned on) {
     return __hiloint2double(__double2hiint(x) ^ (int)(on << 31), __double2loint(x));
@@ -232,22 +232,26 @@ template <typename C, int SIZE> __device__ __forceinline__ void zero_all(C (&v)[
 #pragma unroll
     for (int r = 0; r < SIZE; ++r) v[r] = C{0, 0};
 }
-// conjugation and scale of the last pass, as store_tile applies them
-template <typename C, int SIZE> __device__ __forceinline__ void finish_all(C (&v)[SIZE], const NatArgs &a) {
+// conjugation and scale of the last pass, as store_tile applies them, and the
+// store: put(r, value) for every point
+template <typename C, int SIZE, typename Put> __device__ __forceinline__ void finish_store(C (&v)[SIZE], const NatArgs &a, const Put &put) {
     using Real = decltype(v[0].x);
     if constexpr (sizeof(Real) == 8) {
 #pragma unroll
         for (int r = 0; r < SIZE; ++r) v[r].y = flip_sign(v[r].y, (a.conj >> 1) & 1);
-#pragma unroll 1
-        for (int turn = a.scaled; turn > 0; --turn) {
+        if (a.scaled) {
 #pragma unroll
-            for (int r = 0; r < SIZE; ++r) v[r] = C{v[r].x * a.scale, v[r].y * a.scale};
+            for (int r = 0; r < SIZE; ++r) put(r, C{v[r].x * a.scale, v[r].y * a.scale});
+            asm volatile("" ::: "memory");  // (the two blocks' stores are not merged)
+            return;
         }
     } else if ((a.conj & 2) || a.scaled) {
         const Real sc = (Real)a.scale, sy = (a.conj & 2) ? -sc : sc;
 #pragma unroll
         for (int r = 0; r < SIZE; ++r) v[r] = C{v[r].x * sc, v[r].y * sy};
     }
+#pragma unroll
+    for (int r = 0; r < SIZE; ++r) put(r, v[r]);
 }
 
 // ------------------------------------------------------------------ columns
@@ -339,10 +343,8 @@ template <typename Real, int N, int PI, bool LOOP> struct ColParts {
 #pragma unroll
                 for (int r = 0; r < SIZE; ++r) buf[(at[i] + r * D) * COLS + col] = v[i][r];
             } else if (ok) {
-                finish_all(v[i], a);
                 C *p = dst + (int64_t)k[i] * a.stride;
-#pragma unroll
-                for (int r = 0; r < SIZE; ++r) p[(int64_t)digits_out<N, STAGES, COUNT>(r) * a.stride] = v[i][r];
+                finish_store(v[i], a, [&](int r, C x) { p[(int64_t)digits_out<N, STAGES, COUNT>(r) * a.stride] = x; });
             }
         }
         if constexpr (!LAST) {
@@ -498,10 +500,8 @@ template <typename Real, int N, int PI, bool LOOP> struct RowParts {
 #pragma unroll
                 for (int r = 0; r < SIZE; ++r) buf[line[i] * RC::RS + RC::pad(at[i] + r * D)] = v[i][r];
             } else {
-                finish_all(v[i], a);
                 C *dst = out + line[i] * N + k[i];
-#pragma unroll
-                for (int r = 0; r < SIZE; ++r) dst[digits_out<N, STAGES, COUNT>(r)] = v[i][r];
+                finish_store(v[i], a, [&](int r, C x) { dst[digits_out<N, STAGES, COUNT>(r)] = x; });
             }
         }
         if constexpr (!LAST) {
@@ -537,9 +537,7 @@ __device__ __forceinline__ void nat_row_tile(const C *in, C *out, C *buf, const 
         for (int r = 0; r < N; ++r) v[r] = row[r];
         load_conj(v, a);
         PartStages<Real, N, true, 0>::run(v, tw);
-        finish_all(v, a);
-#pragma unroll
-        for (int r = 0; r < N; ++r) row[digits_out<N, 0, Cfg::parts.count[0]>(r)] = v[r];
+        finish_store(v, a, [&](int r, C x) { row[digits_out<N, 0, Cfg::parts.count[0]>(r)] = x; });
         __syncwarp();
 #pragma unroll
         for (int i = 0; i < N; ++i) {
