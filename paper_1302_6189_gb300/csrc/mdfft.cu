@@ -15,6 +15,7 @@
 #include <map>
 #include <mutex>
 #include <new>
+#include <set>
 #include <string>
 #include <vector>
 
@@ -381,6 +382,23 @@ bool same_plan(const mdfft::RadixPlan &a, const mdfft::RadixPlan &b) {
     return true;
 }
 
+// Loads kernel fn on the current device, so that its first launch does not (the
+// first execution of a plan then takes 0.1 ms, not 0.8); once per process and
+// device, as the query takes about a microsecond of every plan's creation.
+cudaError_t load_kernel(const void *fn) {
+    static std::mutex mutex;
+    static std::set<std::pair<int, const void *>> loaded;
+    int dev = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e != cudaSuccess) return e;
+    std::lock_guard<std::mutex> lock(mutex);
+    if (loaded.count({dev, fn})) return cudaSuccess;
+    cudaFuncAttributes attr;
+    e = cudaFuncGetAttributes(&attr, fn);
+    if (e == cudaSuccess) loaded.insert({dev, fn});
+    return e;
+}
+
 // The launches of an execution that keeps the natural layout: one per axis
 // longer than 1, in the order of the passes.  None (the pass kernels run) for
 // the tensor-core dtypes, spectra left in the last layout, plans that ask
@@ -407,8 +425,7 @@ mdfft_status build_nat(mdfft_plan_s *p) {
         op.args.nlines = (uint32_t)lines;
         op.args.stride = stride[f];
         op.args.fd = mdfft::fastdiv_make((uint32_t)stride[f]);
-        cudaFuncAttributes loaded;  // (loads the kernel now: the first execution took 0.8 ms instead of 0.1)
-        cudaError_t e = cudaFuncGetAttributes(&loaded, op.k.fn);
+        cudaError_t e = load_kernel(op.k.fn);
         if (e == cudaSuccess && op.k.smem > 48 * 1024)
             e = cudaFuncSetAttribute(op.k.fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)op.k.smem);
         if (e != cudaSuccess) return cuda_fail(e, "axis kernel");
