@@ -9,7 +9,12 @@ no L2 flush is needed between steps.
 
 value = algorithmic bytes / device time, the algorithmic bytes of one
 transform being 2 * M * T * 8 (M fused passes, each reading and writing the
-array once; the transposes are inside the passes).
+array once; the transposes are inside the passes).  Two neighbouring axes may
+share a launch and its trip through HBM: pct_hbm_peak counts the trips made.
+
+stdout is the one JSON line; the studies behind it (every order, complex128,
+4-D and 5-D grids, precision, decompositions, serving) go to stderr as a second
+JSON line.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 
@@ -39,7 +44,7 @@ if ROOT not in sys.path:
 METRIC = "M-D FFT GB/s & % HBM peak vs plain; served FFT/s, p50/p99 at stated error"
 SHAPE = (256, 256, 256)
 P_DEFAULT = 4096
-PROFILE = os.path.join(ROOT, "profiles", "fft_pass_256cubed_c64.md")
+PROFILE = os.path.join(ROOT, "profiles", "fft_axes_256cubed_c64.md")
 # everything the profiled kernels are compiled from: every CUDA source and
 # header of the library (the autotuner may pick any variant), and the build
 # script that holds the nvcc flags
@@ -59,8 +64,8 @@ def parse_args():
     ap.add_argument("--no-extra", action="store_true", help="skip the per-order / complex128 table")
     ap.add_argument("--no-cpu", action="store_true", help="skip the CPU oracle baseline")
     ap.add_argument("--profile-case", action="store_true",
-                    help="one warm-up and one profiled forward transform of a batch of 256^3 volumes "
-                         "(3 + 3 pass launches), for ncu captures")
+                    help="one warm-up and one profiled forward transform of a batch of 256^3 volumes, "
+                         "for ncu captures")
     ap.add_argument("--profile-batch", type=int, default=8, help="volumes per launch in --profile-case")
     ap.add_argument("--profile-dtype", default="c64", choices=["c64", "c128", "c64_tc_fp16", "c64_tc_bf16"])
     ap.add_argument("--profile-shape", default="256,256,256", help="grid of --profile-case, e.g. 64,64,64,64")
@@ -74,7 +79,7 @@ def parse_args():
     return ap.parse_args()
 
 
-PROFILE_C128 = os.path.join(ROOT, "profiles", "fft_pass_256cubed_c128.md")
+PROFILE_C128 = os.path.join(ROOT, "profiles", "fft_axes_256cubed_c128.md")
 
 
 def fp64_peak(dev):
@@ -440,7 +445,6 @@ def run_ours(args):
         del ref
 
     clocks = ClockSampler(local)
-    plan.set_timing(True)
     clocks.start()
     barrier(world)
     torch.cuda.synchronize(dev)
@@ -456,6 +460,10 @@ def run_ours(args):
     barrier(world)
     clk = clocks.stop()
     ms = t0.elapsed_time(t1)
+    # per-pass times in steps of their own: the events between the launches take time
+    plan.set_timing(True)
+    for _ in range(max(3, min(args.steps, 20))):
+        step()
     pass_ms, n_timed = plan.pass_times()
     plan.set_timing(False)
     ms_max = max_over_ranks(ms, world)
@@ -467,7 +475,7 @@ def run_ours(args):
     # two neighbouring axes may share a launch and its trip through HBM: the
     # roofline counts the launches an execution makes, one read and write each
     launches = plan.launches()
-    avg_launch_ms = sum(pass_ms) / launches
+    avg_launch_ms = ms / (2 * args.steps * launches)
     achieved = launch_bytes / (avg_launch_ms * 1e-3) / 1e9
     traffic = profile_traffic()
     # the bound the redistribution's access pattern puts on a pass: the same
@@ -517,27 +525,25 @@ def run_ours(args):
         "metric": METRIC, "value": round(value, 2), "unit": "GB/s", "n_gpus": world, "steps": args.steps,
         "warmup": args.warmup, "ms_per_step": round(ms_max / args.steps, 4), "higher_is_better": True,
         "scaling": "weak", "vs_baseline": None, "dtype": "f32", "data": "synthetic",
-        "pct_hbm_peak": round(100.0 * value / world / peak, 1),
+        # HBM bytes of the trips made (value counts M trips per transform)
+        "pct_hbm_peak": round(100.0 * achieved / peak, 1),
         "nominal_gflops": round(world * args.steps * 2 * B * 5.0 * T * math.log2(T) / (ms_max * 1e-3) / 1e9, 1),
         "forward_rel_l2_vs_c128": fwd_err,
         "config": {"workload": "3-D complex64 FFT 256x256x256, forward + normalised inverse, batch of "
                                f"{B} distinct volumes per step",
-                   "P": P, "order": format_order(order, 3), "regimes": comm["regime"],
-                   "comm_points_total": comm["total"], "l2": "inputs larger than L2 (8 x 128 MiB per step)",
+                   "P": P, "order": format_order(order, 3), "comm_points_total": comm["total"],
+                   "l2": "inputs larger than L2 (8 x 128 MiB per step)",
                    "parallelism": f"replicas x{world}", "input": "U[-1,1) re/im, seeds 1303..1310",
-                   "roundtrip_rel_l2": err, "autotune_ms_per_pass": {"default": [round(v, 5) for v in tune_before],
-                                                                      "chosen": [round(v, 5) for v in tune_after]},
-                   "passes": tuned},
-        "roofline": {"kernel": "fft_pass_kernel<float,256>" if launches == 3 else
+                   "roundtrip_rel_l2": err, "autotuned": [t["variant"] for t in plan.tuning()]},
+        "roofline": {"kernel": "fft_nat / fft_pass kernels of 256 points" if launches == 3 else
                      "fft_pair_kernel<256> + fft_nat_col_kernel<256>", "bound": "hbm", "achieved": round(achieved, 1),
                      "peak": peak, "peak_kind": peak_kind, "unit": "GB/s", "frac": round(achieved / peak, 4),
                      "traffic": traffic, "algorithmic_bytes_per_launch": launch_bytes,
-                     "avg_launch_ms": round(avg_launch_ms, 5), "launches_timed": n_timed * launches, "hbm_trips_per_transform": launches,
-                     "pattern_bound_gbs": round(pattern_gbs, 1), "frac_of_pattern": round(achieved / pattern_gbs, 4),
-                     "pass_ms": [round(v, 5) for v in pass_ms],
-                     # ncu DRAM bytes of the M passes over the bytes of one full-array read + write
-                     "full_array_passes_per_transform": None if traffic is None else
-                     round(len(shape) * traffic / launch_bytes, 3)},
+                     "avg_launch_ms": round(avg_launch_ms, 5), "launches_timed": args.steps * 2 * launches,
+                     "hbm_trips_per_transform": launches,
+                     # ncu DRAM bytes of an execution's launches over the bytes of one full-array read + write
+                     "full_array_trips_by_ncu": None if traffic is None else
+                     round(launches * traffic / launch_bytes, 3)},
         "cpu_baseline": cpu,
         "e2e": {"value": round(e2e_value, 2), "unit": "GB/s", "h2d_bytes_per_step": 2 * B * T * elem,
                 "d2h_bytes_per_step": 2 * B * T * elem, "steps": e_steps, "roundtrip_rel_l2": e2e_err,
@@ -547,7 +553,13 @@ def run_ours(args):
         "kernel_source_sha256": kernel_hash(),
     }
     if extra is not None:
-        line["extra"] = extra
+        extra["headline"] = {"pass_ms": [round(v, 5) for v in pass_ms], "pass_ms_executions": n_timed,
+                             "autotune_ms_per_pass": {"default": [round(v, 5) for v in tune_before],
+                                                      "chosen": [round(v, 5) for v in tune_after]},
+                             "passes": tuned, "regimes": comm["regime"],
+                             # the redistributing passes' own data movement, without the butterflies
+                             "pattern_bound_gbs_of_the_passes": round(pattern_gbs, 1)}
+        print(json.dumps({"extra": extra}), file=sys.stderr, flush=True)
     print(json.dumps(line), flush=True)
     barrier(world)
 
@@ -653,7 +665,8 @@ def chunk_order_study(dev, x, P, reps=10):
     out = {"note": f"{B} volumes per launch, forward, {reps} reps, default kernel for both"}
     with Plan(SHAPE, P, order, "c64", batch=B) as pl:
         want = pl.exec(x).clone()
-        base = pl.tuning()
+        # (the pass kernels of the plan as made, not its axis launches)
+        base = [dict(t, variant="passes") for t in pl.tuning()]
         for name, tuning in (("output_runs", base),
                              ("input_chunk_per_cta", [dict(t, tile_g=16, tile_h=1, tile_order=1) for t in base])):
             pl.set_tuning(tuning)
@@ -668,7 +681,6 @@ def chunk_order_study(dev, x, P, reps=10):
             out[name] = {"gbs_per_pass": [round(2 * B * T * 8 / (m * 1e-3) / 1e9, 1) for m in pass_ms],
                          "ctas": [d["ctas"] for d in pl.describe()], "store_axis": [d["store_axis"] for d in pl.describe()],
                          "same_bits": bool(torch.equal(y, want))}
-        pl.set_tuning(base)
     return out
 
 
@@ -752,9 +764,8 @@ def dist_study(dev, x0, P, reps=5):
 
 def small_study(dev, reps=2000):
     """The 32^3 complex128 configuration (P = 4, order abc->cab->cba), forward
-    + normalised inverse per call pair: microseconds per pair with the M pass
-    launches issued one by one (mdfft_exec) and replayed from a captured
-    CUDA graph (mdfft_exec_graph)."""
+    + normalised inverse per call pair: microseconds per pair through mdfft_exec
+    and mdfft_exec_graph (the same axis launches for this plan)."""
     import numpy as np
     import torch
 
@@ -781,7 +792,7 @@ def small_study(dev, reps=2000):
             out["graph_us" if graph else "direct_us"] = round(a.elapsed_time(b) * 1e3 / reps, 2)
         err = float((torch.linalg.vector_norm(z - x) / torch.linalg.vector_norm(x)).item())
     out["roundtrip_rel_l2"] = err
-    out["note"] = "forward + normalised inverse, 6 pass launches or 2 graph launches per pair"
+    out["note"] = "forward + normalised inverse, 6 launches per pair"
     return out
 
 
@@ -817,7 +828,6 @@ def md_study(dev, reps=10):
                     tuning = [dict(t, radix=d["radix"]) for t, d in zip(pl.tuning(), pl.describe())]
                     for _ in range(3):
                         pl.exec(x, y)
-                    pl.set_timing(True)
                     a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
                     a.record()
                     for _ in range(reps):
@@ -825,8 +835,12 @@ def md_study(dev, reps=10):
                     b.record()
                     torch.cuda.synchronize(dev)
                     ms = a.elapsed_time(b) / reps
+                    launches = pl.launches()
+                    pl.set_timing(True)  # (timed executions run a batch axis by axis, in place of groups that L2 holds)
+                    for _ in range(reps):
+                        pl.exec(x, y)
                     pass_ms, _ = pl.pass_times()
-                    trips = min(pl.launches(), M)  # (timed executions run a batch axis by axis)
+                    trips = min(launches, M)
                 name = f"{'x'.join(map(str, shape))} P={P} {'worst' if want else 'best'}"
                 out[name] = {"order": format_order(order, M), "comm_points": amount,
                              "gbs": round(2 * M * T * 8 * B / (ms * 1e-3) / 1e9, 1),
@@ -838,7 +852,7 @@ def md_study(dev, reps=10):
                                            "or the ring kernel (movement) does, with the pass's tiles where they "
                                            "fit that kernel's CTA, else its default tiling; they bound those "
                                            "kernels, not the one- or two-threads-per-line ones",
-                             "hbm_trips_per_transform": trips,
+                             "launches": launches, "hbm_trips_of_the_timed_passes": trips,
                              "roofline": pass_roofline(2 * B * T * 8 * trips / M, pass_ms, MD_PROFILES.get(name))}
     return out
 
@@ -990,7 +1004,7 @@ def precision_study(dev, with_oracle=True):
 
 def profile_case(args):
     """Two forward transforms of a batch of volumes with the planner's best
-    order (M + M pass launches: a warm-up, then the profiled ones, inside the
+    order (a warm-up, then the profiled one, inside the
     NVTX range "profiled"); with --profile-tune the plan is autotuned first."""
     import numpy as np
     import torch
@@ -1014,22 +1028,22 @@ def profile_case(args):
         if args.profile_tuning:
             t = json.loads(args.profile_tuning)
             plan.set_tuning([dict(e) for e in t] if isinstance(t, list) else [dict(t) for _ in shape])
-        plan.exec(x, y)  # warm-up: launches 1..M (after any autotuning)
+        plan.exec(x, y)  # warm-up (after any autotuning)
         torch.cuda.synchronize()
         torch.cuda.nvtx.range_push("profiled")
-        plan.exec(x, y)  # profiled: the next M launches
+        plan.exec(x, y)
         torch.cuda.synchronize()
         torch.cuda.nvtx.range_pop()
         plan.check()
         print(json.dumps({"profile_case": f"{B} x {'x'.join(map(str, shape))} {args.profile_dtype} forward",
-                          "order": plan.order_str(), "tuning": plan.tuning(), "passes": plan.describe()}))
+                          "order": plan.order_str(), "launches": plan.launches(), "tuning": plan.tuning()}))
 
 
 def serving_study(dev, n=2000, budget=40e9):
     """2000 Poisson arrivals: 80 % 3-D requests with axes from {48..192}, 20 %
     32^4, complex64 forward, 40 GB HBM admission budget.  The batched server
-    (one graph launch of one persistent kernel per step) against plain
-    per-request mdfft_exec launches of the same kernels, at arrival rates
+    (one graph launch per step, a kernel per line length and kind) against plain
+    per-request mdfft_exec launches of the axis kernels, at arrival rates
     0.5, 0.8 and 1.0 times the server's saturated throughput X.  Latency is
     arrival (host clock) to completion (CUDA event), both from one zero."""
     import numpy as np
@@ -1098,7 +1112,7 @@ def serving_study(dev, n=2000, budget=40e9):
     with Server(int(budget), max_inflight=512, P=64) as srv:
         for _ in range(2):  # plans, graphs and clocks warm
             run_server(srv, zero)
-        # autotune the persistent grid (whole multiples of the SM count) and the
+        # autotune the kernels' CTAs (whole multiples of the SM count) and the
         # number of steps in flight, on the saturated load (the tiles dealt to a
         # CTA at a time stay at the default maximum of 4: larger chunks raise the
         # saturated rate a little but double the latency at 0.8 X)
@@ -1131,7 +1145,7 @@ def serving_study(dev, n=2000, budget=40e9):
         out["server_stats"] = srv.stats()
     for pl in plans.values():
         pl.close()
-    out["results"] = "identical kernels and tiles in both arms (tests: bit-equal to mdfft_exec)"
+    out["results"] = "the same butterflies in both arms (tests: bit-equal to mdfft_exec)"
     return out
 
 
