@@ -137,7 +137,8 @@ mdfft_status mdfft_plan(mdfft_plan_t *out, int M, const int64_t N[], int64_t P, 
  * plan's workspace is that size too.  Each pass is one launch over the tiles
  * of every transform of the batch (the batch is the outermost tile axis), so
  * the partly filled last wave of CTAs is paid once per pass, not once per
- * transform.  Counted executions add the amounts of all transforms; the
+ * transform; axis launches cover the batch, or groups of its transforms that
+ * L2 holds (mdfft_launches_per_exec).  Counted executions add the amounts of all transforms; the
  * amounts of mdfft_comm_volume are per transform.  batch * T must not exceed
  * 2^40 (E_ARG).
  */
@@ -148,6 +149,9 @@ mdfft_status mdfft_plan_batched(mdfft_plan_t *out, int M, const int64_t N[], int
  * mdfft_exec -- run the plan: M fused passes, pass s doing the 1-D FFTs along
  * the last axis of layout s (Fig. 4, steps 1..M) and storing straight into
  * layout s+1 (the transposes of Fig. 4; the last one gives natural order).
+ * Plans that have axis launches (mdfft_launches_per_exec) transform the same
+ * axes in the same order without moving the data between layouts, in place on
+ * out_dev after the first, with the same bits.
  *   in_dev, out_dev  device arrays of N_1 ... N_M elements of the plan's
  *                    complex type, 16-byte aligned; in_dev is not modified
  *                    unless in_dev == out_dev (needs MDFFT_PLAN_INPLACE);
@@ -326,7 +330,9 @@ mdfft_status mdfft_exec_host(mdfft_plan_t plan, const void *in_host, void *out_h
 
 /* Launch shape of pass s: line length, tile (lines along the tile axes g and
  * h), threads per CTA, CTAs, bytes of shared memory, the radix plan of the
- * 1-D FFTs and the tile order.  Host information only. */
+ * 1-D FFTs and the tile order.  Host information only.  It is the pass kernel's
+ * shape, also where executions run axis launches in its place
+ * (mdfft_launches_per_exec); counted executions always run the pass kernels. */
 typedef struct {
     int64_t line_length;
     int tile_g, tile_h, threads, smem_bytes;
@@ -476,9 +482,11 @@ mdfft_status mdfft_workspace_size(mdfft_plan_t plan, size_t *bytes);
 /* Number of kernel launches one mdfft_exec makes: M with the pass kernels,
  * else at most one per axis longer than 1 (neighbouring axes of 64, 128 or 256
  * points of a complex64 array of 96 MB and more share one), per group of
- * transforms of a batch that L2 holds (64 MB): complex64 and complex128 plans with the
- * default launch choices transform the axes in place, in the natural layout
- * (complex128 unless an axis is 192, 384 or 512). */
+ * transforms of a batch that L2 holds (64 MB; while pass timing is on, the whole
+ * batch): complex64 and complex128 plans with the default launch choices
+ * (mdfft_plan_tuning) and natural output, without MDFFT_PLAN_PERSISTENT,
+ * transform the axes in place, in the natural layout (complex128 unless an axis
+ * is 192, 384 or 512). */
 mdfft_status mdfft_launches_per_exec(mdfft_plan_t plan, int *launches);
 
 /* Is line length n built into this library for dtype dt?  1 yes, 0 no. */
@@ -492,9 +500,10 @@ mdfft_status mdfft_destroy(mdfft_plan_t plan);
  *
  * A server owns a plan per shape (planner's best order for P virtual
  * processes, complex64), a device arena for the workspaces of the requests
- * in flight, and a CUDA graph per table slot.  mdfft_server_step() admits
- * queued requests first come first served while the HBM budget (each request
- * is charged input + output + workspace = 3 T 8 bytes) and the slot count
+ * in flight, and a CUDA graph per table slot, made with the server.
+ * mdfft_server_step() admits queued requests first come first served while the
+ * HBM budget (each request is charged input + output + workspace = 3 T 8 bytes,
+ * the workspace also where its axis launches do not touch it) and the slot count
  * allow, then launches -- as one graph launch -- the next axis of every
  * request in flight, whatever its shape, in the order of the plan's passes.  A
  * request that arrives while others are on the GPU joins at the next step; it

@@ -32,11 +32,16 @@
 // launches together: N x N planes), rows and columns now: N = 24 3,000 -> 6,070,
 // 32 4,040 -> 6,020, 96 4,130 -> 5,180, 160 3,940 -> 5,090, 256 5,520 -> 5,960,
 // 512 4,610 -> 5,180; whole transforms: 24^5 170 -> 76 us (64 MB, in L2), 256^3
-// 142 -> 121 us (108 with fft_pair.cuh), 512^3 1,190 -> 1,056 us.
+// 142 -> 121 us (109 with fft_pair.cuh), 512^3 1,190 -> 1,060 us.  Counters
+// (single precision): 256-point columns 74 % of the DRAM rate and 48 % of the
+// load/store data pipe; 24-point rows 90 % of that pipe, their columns 60 %;
+// 512-point rows 79 % of it at 85 % of the DRAM rate, their columns 30 warps per
+// SM (63 registers) at 70 %; 240-point columns 19 warps (80 registers).
 // Double precision: the FP64 units (a warp instruction holds one for 64
 // cycles), so lanes must not idle and small grids need many short-lived warps
-// spread over the SMs: 32^3 25.6 -> 15.9 us, 64^3 44.2 -> 34.5, 128^3 274 -> 256,
-// 48 x 48 planes (2^22 points) 390 -> 317, 256 x 256 399 -> 386.
+// spread over the SMs: 32^3 25.6 -> 14.9 us, 64^3 44.2 -> 32.8, 128^3 274 -> 245,
+// 48 x 48 planes (2^22 points) 390 -> 270, 256 x 256 399 -> 371; 256^3 runs 22.25
+// FP64 instructions per point and axis in 2,121 us, their issue time being 2,119.
 #pragma once
 
 #include "nat_args.h"
@@ -446,9 +451,10 @@ template <typename Real, int N> struct RowCfg {
     static constexpr int THREADS = sizeof(Real) == 8 ? (LINES * Cfg::TL + 31) / 32 * 32 : LINES * Cfg::TL;
     static_assert(THREADS <= 1024, "CTA shape");
     static constexpr size_t SMEM = (size_t)LINES * RS * sizeof(C);
-    // registers for 40 warps per SM (48 a thread; 32 warps with a 15-point part,
-    // 5 or 6 CTAs with a line of 20 points and more in a thread): uncapped the
-    // compiler spends 60 to 110 on the same code and the warps are missed
+    // registers for 40 warps per SM (48 a thread; 32 warps with a 15-point part
+    // or a multiple of 80 points, whose parts need more; 6 CTAs where a thread
+    // holds a line of 20 points): uncapped the compiler spends 60 to 110 on the
+    // same code and the warps are missed
     static constexpr int MINB = sizeof(Real) == 8      ? 1
                                 : Cfg::parts.n == 1    ? (N >= 20 ? 6 : 1)
                                 : Cfg::parts.max == 15 || N % 80 == 0 ? 1024 / THREADS

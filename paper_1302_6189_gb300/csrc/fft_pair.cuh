@@ -20,11 +20,13 @@
 // that what it added to any counter comes before the zeroes.  (After complete waits the B
 // tiles' acquires order this too; after one that gave up nothing else does.)
 //
-// What bounds it: the shared-memory and load/store pipe of the two axes (27 to
-// 31 us per axis and 2^24 points at 256 points, where a trip through HBM takes
-// 38); both operations together take less than two trips, not one.  Whole
-// transforms, one launch per axis before: 256^3 121 -> 108 us, 256^3 x 8 there and
-// back 1,862 -> 1,637 us, 64^4 x 4 620 -> 536 us.
+// What bounds it: the instructions of the two axes (27 to 31 us per axis and 2^24
+// points at 256 points, where a trip through HBM takes 38; over the launch 60 %
+// of the load/store data pipe and 58 % of the issue slots busy, most stalled
+// warps at the CTA barriers, 50 % of the DRAM rate); both operations together
+// take less than two trips, not one.  Whole transforms, one launch per axis
+// before: 256^3 121 -> 109 us, 256^3 x 8 there and back 1,862 -> 1,639 us, 64^4 x 4
+// 620 -> 539 us.
 //
 // A kernel per length: with every pair of lengths in one kernel (a switch) the
 // tiles ran at 0.6 of this rate.

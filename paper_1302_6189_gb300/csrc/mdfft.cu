@@ -795,8 +795,8 @@ mdfft_status exec_graph_impl(mdfft_plan_t p, const void *in, void *out, int dir,
     mdfft_status cs = check_exec(p, in, out, dir, normalize, nullptr);
     if (cs != MDFFT_OK) return cs;
     // The axis launches follow each other without a gap and need no capture:
-    // launched as they are they take 17.9 us for a 64^3 round trip, as two
-    // graphs 24.2 us (32^3 14.7 / 16.4, 128^3 38.7 / 41.0, 24^5 152.7 / 156.7).
+    // launched as they are they take 14.6 us for a 64^3 round trip, as two
+    // graphs 16.4 us (32^3 14.2 / 16.4, 128^3 30.2 / 36.5, 24^5 149.7 / 154.4).
     if (p->use_nat && !p->nat.empty()) return launch_nat(p, in, out, dir, normalize, st, -1, false);
     mdfft_plan_s::GraphEntry *hit = nullptr;
     for (auto &g : p->graphs)

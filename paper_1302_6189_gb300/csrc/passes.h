@@ -16,7 +16,9 @@
 // Line lengths of the layout-keeping kernels: all of them but 1 (nothing to transform).
 #define MDFFT_NAT_LENGTHS(X) MDFFT_NAT_LENGTHS_C128(X) X(192) X(384) X(512)
 // In double precision without 192, 384 and 512, whose pass kernels measured 1-4 %
-// faster (N x N planes, 2^22 points: 407 / 456 / 465 us against 416 / 462 / 482).
+// faster (N x N planes, 2^22 points: 407 / 456 / 465 us against 416 / 462 / 482,
+// when signs and scale still issued FP64 instructions in the axis kernels; not
+// measured since).  A plan with one such axis runs the pass kernels on all of them.
 #define MDFFT_NAT_LENGTHS_C128(X)                                                                          \
     X(2) X(3) X(4) X(5) X(6) X(8) X(10) X(12) X(15) X(16) X(20) X(24) X(30) X(32) X(40) X(48) X(60) X(64)  \
         X(80) X(96) X(120) X(128) X(160) X(240) X(256) X(320) X(480) X(640) X(768) X(960) X(1024)

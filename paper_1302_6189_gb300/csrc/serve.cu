@@ -420,7 +420,9 @@ mdfft_status mdfft_server_create(mdfft_server_t *out, size_t budget_bytes, int m
     };
     cudaError_t e;
     // workspaces: one T-element array per request in flight; each request is
-    // charged input + output + workspace, so workspaces use at most a third
+    // charged input + output + workspace, so workspaces use at most a third.
+    // Axis launches leave it untouched (they work in place on the output); the
+    // pass kernels of a plan without them need it.
     s->arena_bytes = (budget_bytes / 3 + 255) / 256 * 256;
     if ((e = cudaMalloc(&s->arena_mem, s->arena_bytes)) != cudaSuccess) return bail(cuda_fail(e, "cudaMalloc arena"));
     s->arena.reset(s->arena_bytes);
