@@ -853,13 +853,8 @@ def md_study(dev, reps=10):
                                            "fit that kernel's CTA, else its default tiling; they bound those "
                                            "kernels, not the one- or two-threads-per-line ones",
                              "launches": launches, "hbm_trips_of_the_timed_passes": trips,
-                             "roofline": pass_roofline(2 * B * T * 8 * trips / M, pass_ms, MD_PROFILES.get(name))}
+                             "roofline": pass_roofline(2 * B * T * 8 * trips / M, pass_ms)}
     return out
-
-
-# ncu summaries of the 4-D / 5-D configurations' launches (4 volumes, autotuned plan)
-MD_PROFILES = {"64x64x64x64 P=64 best": os.path.join(ROOT, "profiles", "fft_pass_64x4_c64.md"),
-               "24x24x24x24x24 P=64 best": os.path.join(ROOT, "profiles", "fft_pass_24x5_c64.md")}
 
 
 def movement_bound_ms(pl, s, x, y):
@@ -936,8 +931,7 @@ def decomposition_study(dev):
     return out
 
 
-PRECISION_PROFILES = {"c64": os.path.join(ROOT, "profiles", "fft_pass_512cubed_c64.md"),
-                      "c64_tc_fp16": os.path.join(ROOT, "profiles", "fft_pass_512cubed_tc_fp16.md")}
+PRECISION_PROFILES = {"c64_tc_fp16": os.path.join(ROOT, "profiles", "fft_pass_512cubed_tc_fp16.md")}
 PRECISION_BOUNDS = {"c64": 1e-5, "c64_tc_fp16": 1e-5, "c64_tc_bf16": 1e-4, "c128": 1e-12}
 
 

@@ -476,7 +476,8 @@ mdfft_status mdfft_fp64_rate_probe(double *out_dev, int ctas, int64_t iters, mdf
  * copies, MMA completion). */
 mdfft_status mdfft_plan_check(mdfft_plan_t plan);
 
-/* Device workspace the plan owns, in bytes (0 for host-only plans). */
+/* Device workspace the plan owns, in bytes (0 for host-only plans).  The pass
+ * kernels use it (counted executions and tuned plans too); axis launches do not. */
 mdfft_status mdfft_workspace_size(mdfft_plan_t plan, size_t *bytes);
 
 /* Number of kernel launches one mdfft_exec makes: M with the pass kernels,
