@@ -166,6 +166,13 @@ class ClockSampler:
         except OSError:
             self.proc = None
 
+    def wait_first(self, work, limit_s=3.0):
+        """Keeps the GPU busy with work() until the first sample is there (nvidia-smi
+        takes longer to start than a short timed region lasts)."""
+        end = time.perf_counter() + limit_s
+        while self.proc is not None and os.path.getsize(self.path) == 0 and time.perf_counter() < end:
+            work()
+
     def stop(self):
         if self.proc is None:
             return {"sm_mhz": None, "sm_max_mhz": None, "reasons": ["nvidia-smi unavailable"], "samples": 0}
@@ -446,6 +453,12 @@ def run_ours(args):
 
     clocks = ClockSampler(local)
     clocks.start()
+
+    def busy():
+        step()
+        torch.cuda.synchronize(dev)
+
+    clocks.wait_first(busy)
     barrier(world)
     torch.cuda.synchronize(dev)
     t0 = torch.cuda.Event(enable_timing=True)
